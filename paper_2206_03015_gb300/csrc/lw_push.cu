@@ -1,9 +1,9 @@
 // Boris pusher on the GPU (FP64), the trajectory update of Algorithm 2 ("update
 // trajectory" in the step loop), for the in-situ form of the time-domain path:
 // trajectories are produced one block of steps at a time and deposited at once,
-// so only the current block is ever stored.  The same step, carried out on
-// forward-mode derivative numbers, gives the gradient of a loss of the samples
-// with respect to the initial momenta and the laser's a0 and waist.
+// so only the current block is ever stored.  The same step, differentiated in
+// forward mode, gives the gradient of a loss of the samples with respect to the
+// initial momenta and the laser's a0 and waist.
 //
 // Laser: lowest-order paraxial Gaussian beam polarised along x, propagating
 // along -z, focused at z = 0 and peaking there at t = 0:
@@ -25,193 +25,10 @@ namespace {
 constexpr double kQe = 1.602176634e-19;
 constexpr double kMe = 9.1093837015e-31;
 
-using ::atan;
-using ::cos;
-using ::exp;
-using ::sqrt;
-
-// Forward-mode derivative numbers: a value and its derivatives along N directions.
-template <int N>
-struct Dual {
-    double v;
-    double d[N];
+// Laser constants of the push.
+struct Laser {
+    double omega, k, sigma, E0, zR, w0;
 };
-template <int N>
-__device__ __forceinline__ Dual<N> mk(double v) {
-    Dual<N> r;
-    r.v = v;
-#pragma unroll
-    for (int i = 0; i < N; ++i) r.d[i] = 0.0;
-    return r;
-}
-template <int N>
-__device__ __forceinline__ Dual<N> operator+(const Dual<N>& a, const Dual<N>& b) {
-    Dual<N> r;
-    r.v = a.v + b.v;
-#pragma unroll
-    for (int i = 0; i < N; ++i) r.d[i] = a.d[i] + b.d[i];
-    return r;
-}
-template <int N>
-__device__ __forceinline__ Dual<N> operator-(const Dual<N>& a, const Dual<N>& b) {
-    Dual<N> r;
-    r.v = a.v - b.v;
-#pragma unroll
-    for (int i = 0; i < N; ++i) r.d[i] = a.d[i] - b.d[i];
-    return r;
-}
-template <int N>
-__device__ __forceinline__ Dual<N> operator-(const Dual<N>& a) {
-    Dual<N> r;
-    r.v = -a.v;
-#pragma unroll
-    for (int i = 0; i < N; ++i) r.d[i] = -a.d[i];
-    return r;
-}
-template <int N>
-__device__ __forceinline__ Dual<N> operator*(const Dual<N>& a, const Dual<N>& b) {
-    Dual<N> r;
-    r.v = a.v * b.v;
-#pragma unroll
-    for (int i = 0; i < N; ++i) r.d[i] = a.d[i] * b.v + a.v * b.d[i];
-    return r;
-}
-template <int N>
-__device__ __forceinline__ Dual<N> operator/(const Dual<N>& a, const Dual<N>& b) {
-    Dual<N> r;
-    r.v = a.v / b.v;
-    const double ib = 1.0 / b.v;
-#pragma unroll
-    for (int i = 0; i < N; ++i) r.d[i] = (a.d[i] - r.v * b.d[i]) * ib;
-    return r;
-}
-template <int N>
-__device__ __forceinline__ Dual<N> operator+(const Dual<N>& a, double b) {
-    Dual<N> r = a;
-    r.v = a.v + b;
-    return r;
-}
-template <int N>
-__device__ __forceinline__ Dual<N> operator+(double a, const Dual<N>& b) { return b + a; }
-template <int N>
-__device__ __forceinline__ Dual<N> operator-(const Dual<N>& a, double b) { return a + (-b); }
-template <int N>
-__device__ __forceinline__ Dual<N> operator-(double a, const Dual<N>& b) { return (-b) + a; }
-template <int N>
-__device__ __forceinline__ Dual<N> operator*(const Dual<N>& a, double b) {
-    Dual<N> r;
-    r.v = a.v * b;
-#pragma unroll
-    for (int i = 0; i < N; ++i) r.d[i] = a.d[i] * b;
-    return r;
-}
-template <int N>
-__device__ __forceinline__ Dual<N> operator*(double a, const Dual<N>& b) { return b * a; }
-template <int N>
-__device__ __forceinline__ Dual<N> operator/(const Dual<N>& a, double b) { return a * (1.0 / b); }
-template <int N>
-__device__ __forceinline__ Dual<N> operator/(double a, const Dual<N>& b) { return mk<N>(a) / b; }
-template <int N>
-__device__ __forceinline__ Dual<N> sqrt(const Dual<N>& a) {
-    Dual<N> r;
-    r.v = sqrt(a.v);
-    const double h = 0.5 / r.v;
-#pragma unroll
-    for (int i = 0; i < N; ++i) r.d[i] = a.d[i] * h;
-    return r;
-}
-template <int N>
-__device__ __forceinline__ Dual<N> exp(const Dual<N>& a) {
-    Dual<N> r;
-    r.v = exp(a.v);
-#pragma unroll
-    for (int i = 0; i < N; ++i) r.d[i] = a.d[i] * r.v;
-    return r;
-}
-template <int N>
-__device__ __forceinline__ Dual<N> cos(const Dual<N>& a) {
-    Dual<N> r;
-    double sn, cs;
-    sincos(a.v, &sn, &cs);
-    r.v = cs;
-#pragma unroll
-    for (int i = 0; i < N; ++i) r.d[i] = -a.d[i] * sn;
-    return r;
-}
-template <int N>
-__device__ __forceinline__ Dual<N> atan(const Dual<N>& a) {
-    Dual<N> r;
-    r.v = atan(a.v);
-    const double h = 1.0 / (1.0 + a.v * a.v);
-#pragma unroll
-    for (int i = 0; i < N; ++i) r.d[i] = a.d[i] * h;
-    return r;
-}
-
-// Laser constants (T = double, or Dual when derivatives along a0 and w0 are carried).
-template <typename T>
-struct LaserT {
-    double omega, k, sigma;
-    T E0, zR, w0;
-};
-using Laser = LaserT<double>;
-
-template <typename T>
-__device__ __forceinline__ void fields(const LaserT<T>& L, const T& x, const T& y, const T& z,
-                                       double t, T& Ex, T& By) {
-    const T zeta = -z;
-    const T w = L.w0 * sqrt(1.0 + (zeta / L.zR) * (zeta / L.zR));
-    const T rho2 = x * x + y * y;
-    const T xi = t + z * kInvC0;
-    const T env = exp(-rho2 / (w * w)) * exp(-(xi * xi) / (2.0 * L.sigma * L.sigma));
-    const T phase =
-        L.omega * xi + L.k * rho2 * zeta / (2.0 * (zeta * zeta + L.zR * L.zR)) - atan(zeta / L.zR);
-    Ex = L.E0 * (L.w0 / w) * env * cos(phase);
-    By = -Ex * kInvC0;
-}
-
-// The sample at (r, u): beta = u / gamma and the Lorentz-force beta_dot.
-template <typename T>
-__device__ __forceinline__ void sample(const LaserT<T>& L, double qm, const T r[3], const T u[3],
-                                       double t, T b[3], T a[3]) {
-    const T gam = sqrt(1.0 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-    b[0] = u[0] / gam;
-    b[1] = u[1] / gam;
-    b[2] = u[2] / gam;
-    T Ex, By;
-    fields(L, r[0], r[1], r[2], t, Ex, By);
-    // E = (Ex, 0, 0), B = (0, By, 0): beta x B = (-b_z By, 0, b_x By)
-    const T bE = b[0] * Ex;
-    const T f = qm / (gam * kC0);
-    a[0] = f * (Ex + kC0 * (-b[2] * By) - b[0] * bE);
-    a[1] = f * (-b[1] * bE);
-    a[2] = f * (kC0 * (b[0] * By) - b[2] * bE);
-}
-
-// One Boris step from time ti: drift dt/2, kick with the fields at the midpoint, drift.
-template <typename T>
-__device__ __forceinline__ void boris_step(const LaserT<T>& L, double qm, double dt, double ti,
-                                           T x[3], T v[3]) {
-    const double eps = qm * dt / (2.0 * kC0);
-    T gam = sqrt(1.0 + v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
-    const T rh[3] = {x[0] + 0.5 * dt * kC0 * v[0] / gam, x[1] + 0.5 * dt * kC0 * v[1] / gam,
-                     x[2] + 0.5 * dt * kC0 * v[2] / gam};
-    T Ex, By;
-    fields(L, rh[0], rh[1], rh[2], ti + 0.5 * dt, Ex, By);
-    const T um[3] = {v[0] + eps * Ex, v[1], v[2]};
-    const T gm = sqrt(1.0 + um[0] * um[0] + um[1] * um[1] + um[2] * um[2]);
-    const T tv = qm * dt / (2.0 * gm) * By;   // t vector = (0, tv, 0)
-    // u' = um + um x t ; s = 2 t / (1 + t^2) ; u+ = um + u' x s
-    const T up[3] = {um[0] - um[2] * tv, um[1], um[2] + um[0] * tv};
-    const T sv = 2.0 * tv / (1.0 + tv * tv);
-    v[0] = um[0] - up[2] * sv + eps * Ex;
-    v[1] = um[1];
-    v[2] = um[2] + up[0] * sv;
-    gam = sqrt(1.0 + v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
-    x[0] = rh[0] + 0.5 * dt * kC0 * v[0] / gam;
-    x[1] = rh[1] + 0.5 * dt * kC0 * v[1] / gam;
-    x[2] = rh[2] + 0.5 * dt * kC0 * v[2] / gam;
-}
 
 // ------------------------------------------------------------------ the push
 //
@@ -234,7 +51,7 @@ __device__ __forceinline__ void boris_step(const LaserT<T>& L, double qm, double
 // and of the kick adds rounded squares, gamma of the second half drift fuses them).  A square
 // root and the quotients by it share one reciprocal square root, with a residual correction
 // for each correctly rounded result; zeta/zR uses the host's reciprocal the same way.  Only
-// the samples' beta and beta_dot use a shorter form (sample_beam()).
+// the samples' beta and beta_dot use a shorter form (beam_value()).
 // One warp per 32 electrons doing all of it took 15.7 us per step (1,500 electrons, 10,000
 // steps: 157 ms); cut this way it takes 5.0 us (50 ms).
 struct Beam {
@@ -243,22 +60,27 @@ struct Beam {
     double E0;
 };
 
-// E_x of fields() in the form
-//   E0 exp(-rho^2/(w0^2 q) - xi^2/(2 sigma^2)) (cos phi + s sin phi) / q,
+// E_x / E0 in the form
+//   U = exp(-rho^2/(w0^2 q) - xi^2/(2 sigma^2)) (cos phi + s sin phi) / q,
 //   s = zeta/zR, q = 1 + s^2, phi = omega xi + k rho^2 s / (2 zR q), xi = t + z/c0,
 // from w^2 = w0^2 q and cos(phi - atan s) = (cos phi + s sin phi) / sqrt(q): one exponential,
 // one reciprocal and no arc tangent or square root.
-__device__ __forceinline__ double sample_beam(const Beam& B, double x, double y, double z,
-                                              double t) {
-    const double s = -z * B.inv_zR;
-    const double iq = 1.0 / fma(s, s, 1.0);
-    const double g = fma(x, x, y * y) * iq;
-    const double xi = fma(z, kInvC0, t);
-    const double env = exp(-fma(g, B.inv_w02, xi * xi * B.inv_2s2));
-    double sn, cs;
-    sincospi(fma(B.om_pi, xi, B.kz_pi * (g * s)), &sn, &cs);
-    return B.E0 * iq * env * fma(s, sn, cs);
+struct BeamValue {
+    double s, iq, g, xi;    // zeta/zR, 1/q, rho^2/q, xi
+    double A, sn, cs;       // exp(...)/q, sin phi, cos phi
+};
+__device__ __forceinline__ BeamValue beam_value(const Beam& B, double x, double y, double z,
+                                                double t) {
+    BeamValue b;
+    b.s = -z * B.inv_zR;
+    b.iq = 1.0 / fma(b.s, b.s, 1.0);
+    b.g = fma(x, x, y * y) * b.iq;
+    b.xi = fma(z, kInvC0, t);
+    b.A = b.iq * exp(-fma(b.g, B.inv_w02, b.xi * b.xi * B.inv_2s2));
+    sincospi(fma(B.om_pi, b.xi, B.kz_pi * (b.g * b.s)), &b.sn, &b.cs);
+    return b;
 }
+__device__ __forceinline__ double beam_unit(const BeamValue& b) { return b.A * fma(b.s, b.sn, b.cs); }
 
 // n / d correctly rounded, given the reciprocal r of d to an ulp (residual correction; the
 // error left before the last rounding is 2^-105 of the quotient)
@@ -432,7 +254,8 @@ __global__ void __launch_bounds__(kPushThreads)
             const double b0 = u0 * ig, b1 = u1 * ig, b2 = u2 * ig;
             // E = (Ex, 0, 0), c0 B = (0, -Ex, 0):
             // E + c0 beta x B - beta (beta . E) = Ex (1 + b_z - b_x^2, -b_x b_y, -b_x (1 + b_z))
-            const double f = f0 * ig * sample_beam(B, x, y, z, t), g = f * b0, h = 1.0 + b2;
+            const double f = f0 * ig * (B.E0 * beam_unit(beam_value(B, x, y, z, t)));
+            const double g = f * b0, h = 1.0 + b2;
             if (k < n_e) {
                 const int64_t o = base + 3 * (int64_t)s;
                 ro[o] = x;
@@ -450,59 +273,289 @@ __global__ void __launch_bounds__(kPushThreads)
     }
 }
 
-// Gradient of a loss L(samples) with respect to each electron's initial momentum u0 and
-// the laser's a0 and w0, by forward-mode differentiation of the push: one thread per
-// (electron, direction) pushes the electron again carrying the derivative of its state
-// along one of u0_x, u0_y, u0_z, a0 and w0 (Dual<1>) and contracts each sample's
-// derivative with dL/d(r, beta, beta_dot) of that sample.  Five threads per electron
-// rather than one thread with all five directions: the push is a sequential FP64 chain
-// per electron, and GB300's FP64 rate per SM sub-partition makes a single warp's
-// instructions slow, so the work is spread over five times as many warps.  Per-electron
-// a0 and w0 parts are added to dL_dlaser with FP64 atomics.
-constexpr int kTan = 5;
-__global__ void push_tangent_kernel(const double* __restrict__ r0, const double* __restrict__ u0,
-                                    int64_t n_e, double t0, double dt, int n_steps, Laser L0,
-                                    double e0_per_a0, double zr_per_w0, double qm,
-                                    const double* __restrict__ g_r, const double* __restrict__ g_b,
-                                    const double* __restrict__ g_a, double* __restrict__ dL_du0,
-                                    double* __restrict__ dL_dlaser) {
-    using D = Dual<1>;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n_e * kTan;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t k = t / kTan;
-        const int dir = (int)(t - k * kTan);   // 0..2: u0 components, 3: a0, 4: w0
-        LaserT<D> L;
-        L.omega = L0.omega;
-        L.k = L0.k;
-        L.sigma = L0.sigma;
-        L.E0 = D{L0.E0, {dir == 3 ? e0_per_a0 : 0.0}};
-        L.zR = D{L0.zR, {dir == 4 ? zr_per_w0 : 0.0}};
-        L.w0 = D{L0.w0, {dir == 4 ? 1.0 : 0.0}};
-        D x[3], v[3];
+// ------------------------------------------------------------------ its gradient
+//
+// Gradient of a loss L(samples) with respect to each electron's initial momentum u0 and the
+// laser's a0 and w0, in forward mode: the derivative of an electron's state along u0_x, u0_y,
+// u0_z, a0 and w0 is carried through the push and contracted with dL/d(r, beta, beta_dot) of
+// every sample.  Bound as the push is: FP64 instructions of the busiest warp.  Everything that
+// the five directions share is computed once per electron, by the warps of a CTA over the same
+// 32 electrons, as a pipeline over the steps with one barrier per step (ring of four slots):
+//   warp 0   the push itself (step n);
+//   warp 1   the sample's adjoint (sample n): dL/d(sample) pulled back to the state and the
+//            laser, W . (dx, du, da0, dw0);
+//   warp 2   directions a0 and w0 (step n - 2), and the gradient of the field at the midpoint
+//            (step n - 1);
+//   warp 3   directions u0_x, u0_y, u0_z (step n - 2).
+// A direction costs 33 operations per step (the step linearised with coefficients from warps 0
+// and 2) and 6 for the contraction.  One thread per electron and direction, each pushing the
+// electron again in derivative numbers, took 26.6 us per step (2,048 electrons x 4,096 steps:
+// 109 ms); this form 4.6 us (19.0 ms).
+
+// Gradient of E_x = E0 U with respect to (x, y, z), and along a0 and w0.
+struct BeamGrad {
+    double x, y, z, a0, w0;
+};
+struct TanLaser {   // constants of the gradient
+    double kz, om_c, inv_s2c, e0_per_a0, two_over_w0;   // k/(2 zR), omega/c0, 1/(sigma^2 c0)
+};
+// With A the amplitude, P = dE/dphi and g = rho^2/q: dE = Cg dg + Cs ds + (P omega - E xi/sigma^2)
+// dxi, where dg = 2 (x dx + y dy)/q - 2 s g ds/q is already part of Cs; zR varies as w0^2.
+__device__ __forceinline__ BeamGrad beam_grad(const Beam& B, const TanLaser& T,
+                                              const BeamValue& b, double x, double y) {
+    const double U = beam_unit(b), E = B.E0 * U, a = B.E0 * b.A;
+    const double P = a * fma(b.s, b.cs, -b.sn);
+    const double Pk = P * T.kz;
+    const double Ew = E * B.inv_w02;
+    const double Cg = fma(Pk, b.s, -Ew);
+    const double Cs = fma(Pk, b.g, fma(a, b.sn, -2.0 * b.s * b.iq * fma(Cg, b.g, E)));
+    const double c2 = 2.0 * Cg * b.iq;
+    BeamGrad G;
+    G.x = c2 * x;
+    G.y = c2 * y;
+    G.z = fma(P, T.om_c, fma(-E * b.xi, T.inv_s2c, -Cs * B.inv_zR));
+    G.a0 = T.e0_per_a0 * U;
+    G.w0 = T.two_over_w0 * fma(Ew, b.g, -b.s * fma(Pk, b.g, Cs));
+    return G;
+}
+
+constexpr int kTanThreads = 128;
+constexpr int kTanSlots = 4;
+// one slot of the ring (doubles per electron)
+enum {
+    kX = 0, kV = 3, kIg = 6,                     // state n (x, u, 1/gamma)
+    kMx = 7, kMy, kBs, kBiq, kBg, kBxi, kBA, kBsn, kBcs,   // midpoint of step n
+    kUm = 16, kTa, kTb, kTr, kRc, kRs, kV0r,     // kick of step n
+    kG = 23,                                     // field gradient of step n (x, y, z, a0, w0)
+    kW = 28,                                     // adjoint of sample n (x, u, a0, w0)
+    kSlotVals = 36
+};
+
+__global__ void __launch_bounds__(kTanThreads)
+    push_tangent_kernel(const double* __restrict__ r0, const double* __restrict__ u0, int64_t n_e,
+                        double t0, double dt, int n_steps, Beam B, TanLaser T, double qm,
+                        const double* __restrict__ g_r, const double* __restrict__ g_b,
+                        const double* __restrict__ g_a, double* __restrict__ dL_du0,
+                        double* __restrict__ dL_dlaser) {
+    __shared__ double s_ring[kTanSlots][kSlotVals][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t k = blockIdx.x * (int64_t)32 + lane;
+    const int64_t kc = k < n_e ? k : n_e - 1;   // lanes past the end repeat the last electron
+    const double kd = 0.5 * dt * kC0, eps = qm * dt / (2.0 * kC0);
+    auto at = [&](int n, int i) -> double& { return s_ring[n & (kTanSlots - 1)][i][lane]; };
+    auto inv_gamma = [](const double (&u)[3]) {
+        return rsqrt(fma(u[2], u[2], fma(u[1], u[1], fma(u[0], u[0], 1.0))));
+    };
+    // warp 0: state of the step; warp 1: the next sample's dL/d(sample)
+    double x[3], v[3], ig = 1.0;
+    double g[9];
+    // warps 2 and 3: state derivatives of up to three directions, their half drifts' delta and sums
+    constexpr int kDirs = 3;
+    double dx[kDirs][3], dv[kDirs][3], de[kDirs][3], acc[kDirs];
+    const int n_dir = warp == 2 ? 2 : 3;
+    if (warp == 0) {
         for (int c = 0; c < 3; ++c) {
-            x[c] = mk<1>(r0[3 * k + c]);
-            v[c] = mk<1>(u0[3 * k + c]);
-            v[c].d[0] = dir == c ? 1.0 : 0.0;
+            x[c] = r0[3 * kc + c];
+            v[c] = u0[3 * kc + c];
+            at(0, kX + c) = x[c];
+            at(0, kV + c) = v[c];
         }
-        double acc = 0.0;
-        const int64_t base = k * (int64_t)(n_steps + 1);
-        auto contract = [&](int64_t o, double tt) {
-            D b[3], a[3];
-            sample(L, qm, x, v, tt, b, a);
-            for (int c = 0; c < 3; ++c)
-                acc = fma(g_r[3 * o + c], x[c].d[0],
-                          fma(g_b[3 * o + c], b[c].d[0], fma(g_a[3 * o + c], a[c].d[0], acc)));
-        };
-        contract(base, t0);
-        for (int s = 0; s < n_steps; ++s) {
-            boris_step(L, qm, dt, t0 + dt * (double)s, x, v);
-            contract(base + s + 1, t0 + dt * (double)(s + 1));
-        }
-        if (dir < 3)
-            dL_du0[3 * k + dir] += acc;
-        else
-            atomicAdd(dL_dlaser + (dir - 3), acc);
+        ig = inv_gamma(v);
+        at(0, kIg) = ig;
     }
+    auto load_g = [&](int n) {   // dL/d(sample n)
+        const int64_t o = 3 * (kc * (int64_t)(n_steps + 1) + n);
+        for (int c = 0; c < 3; ++c) {
+            g[c] = g_r[o + c];
+            g[3 + c] = g_b[o + c];
+            g[6 + c] = g_a[o + c];
+        }
+    };
+    if (warp == 1) load_g(0);
+    for (int d = 0; d < kDirs; ++d) {
+        acc[d] = 0.0;
+        for (int c = 0; c < 3; ++c) {
+            dx[d][c] = de[d][c] = 0.0;
+            dv[d][c] = warp == 3 && d == c ? 1.0 : 0.0;
+        }
+    }
+    __syncthreads();
+    // delta of a half drift, d(K u/gamma) = K/gamma du - K/gamma^3 (u . du) u, at state n
+    auto half_drift = [&](int n) {
+        const double i1 = at(n, kIg), c1 = kd * i1, c2 = c1 * i1 * i1;
+        const double w0 = at(n, kV), w1 = at(n, kV + 1), w2 = at(n, kV + 2);
+#pragma unroll
+        for (int d = 0; d < kDirs; ++d) {
+            if (d >= n_dir) break;
+            const double w = -c2 * fma(w2, dv[d][2], fma(w1, dv[d][1], w0 * dv[d][0]));
+            de[d][0] = fma(c1, dv[d][0], w * w0);
+            de[d][1] = fma(c1, dv[d][1], w * w1);
+            de[d][2] = fma(c1, dv[d][2], w * w2);
+        }
+    };
+    if (warp >= 2) half_drift(0);
+
+    for (int it = 0; it <= n_steps + 2; ++it) {
+        if (warp == 0) {
+            if (it < n_steps) {   // step it: drift, kick, drift, as the push
+                const double d = kd * ig;
+                const double h0 = fma(v[0], d, x[0]), h1 = fma(v[1], d, x[1]),
+                             h2 = fma(v[2], d, x[2]);
+                const BeamValue b = beam_value(B, h0, h1, h2, fma(dt, (double)it + 0.5, t0));
+                at(it, kMx) = h0;
+                at(it, kMy) = h1;
+                at(it, kBs) = b.s;
+                at(it, kBiq) = b.iq;
+                at(it, kBg) = b.g;
+                at(it, kBxi) = b.xi;
+                at(it, kBA) = b.A;
+                at(it, kBsn) = b.sn;
+                at(it, kBcs) = b.cs;
+                const double e = eps * (B.E0 * beam_unit(b));
+                const double um[3] = {v[0] + e, v[1], v[2]};
+                const double igm = inv_gamma(um);
+                // rotation in the (z, x) plane by theta, tan(theta/2) = tv
+                const double tv = -e * igm;
+                const double rr = 2.0 / fma(tv, tv, 1.0);
+                const double sn = rr * tv, cs = fma(-tv, sn, 1.0);
+                const double v0r = fma(cs, um[0], -sn * v[2]);
+                at(it, kUm) = um[0];
+                at(it, kTa) = -eps * igm;          // dtv = kTa dE - kTb (um . dum)
+                at(it, kTb) = tv * igm * igm;
+                at(it, kTr) = rr;
+                at(it, kRc) = cs;
+                at(it, kRs) = sn;
+                at(it, kV0r) = v0r;
+                v[2] = fma(cs, v[2], sn * um[0]);
+                v[0] = v0r + e;
+                ig = inv_gamma(v);
+                const double d2 = kd * ig;
+                x[0] = fma(v[0], d2, h0);
+                x[1] = fma(v[1], d2, h1);
+                x[2] = fma(v[2], d2, h2);
+                for (int c = 0; c < 3; ++c) {
+                    at(it + 1, kX + c) = x[c];
+                    at(it + 1, kV + c) = v[c];
+                }
+                at(it + 1, kIg) = ig;
+            }
+        } else if (warp == 1) {
+            if (it <= n_steps) {   // sample it: psi = g_r . r + g_b . beta + g_a . beta_dot
+                const double gr[3] = {g[0], g[1], g[2]}, gb[3] = {g[3], g[4], g[5]},
+                             ga[3] = {g[6], g[7], g[8]};
+                if (it < n_steps) load_g(it + 1);
+                const double sx = at(it, kX), sy = at(it, kX + 1), sz = at(it, kX + 2);
+                const double u_0 = at(it, kV), u_1 = at(it, kV + 1), u_2 = at(it, kV + 2);
+                const double i1 = at(it, kIg);
+                const BeamValue b = beam_value(B, sx, sy, sz, fma(dt, (double)it, t0));
+                const BeamGrad G = beam_grad(B, T, b, sx, sy);
+                const double b0 = u_0 * i1, b1 = u_1 * i1, b2 = u_2 * i1, h = 1.0 + b2;
+                // beta_dot = f (h - b0^2, -b0 b1, -b0 h), f = q/(m c0) E / gamma
+                const double fe = qm / kC0 * i1, f = fe * (B.E0 * beam_unit(b));
+                const double m = fma(ga[1], b1, ga[2] * h);
+                const double y = fma(ga[0], fma(-b0, b0, h), -b0 * m);   // dpsi/df
+                const double q = fe * y;                                  // dpsi/dE
+                const double B0 = fma(f, fma(-2.0 * b0, ga[0], -m), gb[0]);
+                const double B1 = fma(-f * b0, ga[1], gb[1]);
+                const double B2 = fma(f, fma(-b0, ga[2], ga[0]), gb[2]);
+                // 1/gamma enters beta = u/gamma and f: d(1/gamma) = -(1/gamma)^2 beta . du
+                const double ki = fma(f, y, fma(B2, b2, fma(B1, b1, B0 * b0)));
+                at(it, kW) = fma(q, G.x, gr[0]);
+                at(it, kW + 1) = fma(q, G.y, gr[1]);
+                at(it, kW + 2) = fma(q, G.z, gr[2]);
+                at(it, kW + 3) = i1 * fma(-ki, b0, B0);
+                at(it, kW + 4) = i1 * fma(-ki, b1, B1);
+                at(it, kW + 5) = i1 * fma(-ki, b2, B2);
+                at(it, kW + 6) = q * G.a0;
+                at(it, kW + 7) = q * G.w0;
+            }
+        } else {
+            if (warp == 2 && it >= 1 && it - 1 < n_steps) {
+                const int n = it - 1;
+                BeamValue b;
+                b.s = at(n, kBs);
+                b.iq = at(n, kBiq);
+                b.g = at(n, kBg);
+                b.xi = at(n, kBxi);
+                b.A = at(n, kBA);
+                b.sn = at(n, kBsn);
+                b.cs = at(n, kBcs);
+                const BeamGrad G = beam_grad(B, T, b, at(n, kMx), at(n, kMy));
+                at(n, kG) = G.x;
+                at(n, kG + 1) = G.y;
+                at(n, kG + 2) = G.z;
+                at(n, kG + 3) = G.a0;
+                at(n, kG + 4) = G.w0;
+            }
+            const int n = it - 2;
+            if (n >= 0) {
+                const double W0 = at(n, kW), W1 = at(n, kW + 1), W2 = at(n, kW + 2);
+                const double W3 = at(n, kW + 3), W4 = at(n, kW + 4), W5 = at(n, kW + 5);
+#pragma unroll
+                for (int d = 0; d < kDirs; ++d) {
+                    if (d >= n_dir) break;
+                    if (warp == 2) acc[d] += at(n, kW + 6 + d);
+                    acc[d] = fma(W0, dx[d][0], fma(W1, dx[d][1], fma(W2, dx[d][2], acc[d])));
+                    acc[d] = fma(W3, dv[d][0], fma(W4, dv[d][1], fma(W5, dv[d][2], acc[d])));
+                }
+                if (n < n_steps) {
+                    const double Gx = at(n, kG), Gy = at(n, kG + 1), Gz = at(n, kG + 2);
+                    const double um = at(n, kUm), ta = at(n, kTa), tb = at(n, kTb);
+                    const double rr = at(n, kTr), cs = at(n, kRc), sn = at(n, kRs);
+                    const double v0r = at(n, kV0r), v1 = at(n, kV + 1), v2 = at(n, kV + 2);
+                    const double v2n = at(n + 1, kV + 2);
+#pragma unroll
+                    for (int d = 0; d < kDirs; ++d) {
+                        if (d >= n_dir) break;
+                        for (int c = 0; c < 3; ++c) dx[d][c] += de[d][c];   // midpoint
+                        double dE = Gx * dx[d][0];
+                        if (warp == 2) dE += at(n, kG + 3 + d);
+                        dE = fma(Gz, dx[d][2], fma(Gy, dx[d][1], dE));
+                        const double dum = fma(eps, dE, dv[d][0]);
+                        const double dot = fma(v2, dv[d][2], fma(v1, dv[d][1], um * dum));
+                        const double dth = rr * fma(ta, dE, -tb * dot);
+                        dv[d][0] = fma(eps, dE, fma(-v2n, dth, fma(-sn, dv[d][2], cs * dum)));
+                        dv[d][2] = fma(v0r, dth, fma(cs, dv[d][2], sn * dum));
+                    }
+                    half_drift(n + 1);
+#pragma unroll
+                    for (int d = 0; d < kDirs; ++d)
+                        for (int c = 0; c < 3; ++c) dx[d][c] += de[d][c];
+                }
+            }
+        }
+        __syncthreads();   // slots it and it + 1 are readable, slot it - 2 is free
+    }
+    if (warp == 3 && k < n_e)
+        for (int c = 0; c < 3; ++c) dL_du0[3 * k + c] += acc[c];
+    if (warp == 2)
+        for (int d = 0; d < 2; ++d) {
+            double a = k < n_e ? acc[d] : 0.0;
+            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if (lane == 0) atomicAdd(dL_dlaser + d, a);
+        }
+}
+
+Laser laser_constants(const lw_laser& l) {
+    Laser L;
+    L.omega = 2.0 * kPi * kC0 / l.lam;
+    L.k = L.omega * kInvC0;
+    L.sigma = l.fwhm / (2.0 * sqrt(log(2.0)));
+    L.E0 = l.a0 * kMe * kC0 * L.omega / kQe;
+    L.zR = kPi * l.w0 * l.w0 / l.lam;
+    L.w0 = l.w0;
+    return L;
+}
+
+Beam beam_constants(const Laser& L) {
+    Beam B;
+    B.inv_zR = 1.0 / L.zR;
+    B.inv_w02 = 1.0 / (L.w0 * L.w0);
+    B.inv_2s2 = 1.0 / (2.0 * L.sigma * L.sigma);
+    B.om_pi = L.omega / kPi;
+    B.kz_pi = L.k / (2.0 * kPi * L.zR);
+    B.E0 = L.E0;
+    return B;
 }
 
 }  // namespace
@@ -520,20 +573,8 @@ extern "C" int lw_boris_push(double* r, double* u, int64_t n_e, double t0, doubl
         !isfinite(t0) || !(mass > 0.0))
         return LW_EINVAL;
     if (!(laser->lam > 0.0) || !(laser->w0 > 0.0) || !(laser->fwhm > 0.0)) return LW_EINVAL;
-    Laser L;
-    L.omega = 2.0 * kPi * kC0 / laser->lam;
-    L.k = L.omega * kInvC0;
-    L.sigma = laser->fwhm / (2.0 * sqrt(log(2.0)));
-    L.E0 = laser->a0 * kMe * kC0 * L.omega / kQe;
-    L.zR = kPi * laser->w0 * laser->w0 / laser->lam;
-    L.w0 = laser->w0;
-    Beam B;
-    B.inv_zR = 1.0 / L.zR;
-    B.inv_w02 = 1.0 / (L.w0 * L.w0);
-    B.inv_2s2 = 1.0 / (2.0 * L.sigma * L.sigma);
-    B.om_pi = L.omega / kPi;
-    B.kz_pi = L.k / (2.0 * kPi * L.zR);
-    B.E0 = L.E0;
+    const Laser L = laser_constants(*laser);
+    const Beam B = beam_constants(L);
     const int blocks = (int)((n_e + 31) / 32);
     push_kernel<<<blocks, kPushThreads, 0, as_stream(stream)>>>(
         r, u, n_e, t0, dt, step0, n_steps, L, B, charge / mass, t_out, r_out, beta_out, bdot_out);
@@ -550,21 +591,16 @@ extern "C" int lw_boris_push_grad(const double* r0, const double* u0, int64_t n_
     if (n_e < 1 || n_steps < 1 || !(dt > 0.0) || !isfinite(t0) || !(mass > 0.0))
         return LW_EINVAL;
     if (!(laser->lam > 0.0) || !(laser->w0 > 0.0) || !(laser->fwhm > 0.0)) return LW_EINVAL;
-    Laser L;
-    L.omega = 2.0 * kPi * kC0 / laser->lam;
-    L.k = L.omega * kInvC0;
-    L.sigma = laser->fwhm / (2.0 * sqrt(log(2.0)));
-    const double e0_per_a0 = kMe * kC0 * L.omega / kQe;
-    L.E0 = laser->a0 * e0_per_a0;
-    L.zR = kPi * laser->w0 * laser->w0 / laser->lam;
-    L.w0 = laser->w0;
-    const double zr_per_w0 = 2.0 * kPi * laser->w0 / laser->lam;
-    // one warp per block: the warps spread over the SMs' sub-partitions
-    const int threads = 32;
-    const int64_t work = n_e * kTan;
-    const int blocks = (int)std::min<int64_t>((work + threads - 1) / threads, 1 << 20);
-    push_tangent_kernel<<<blocks, threads, 0, as_stream(stream)>>>(
-        r0, u0, n_e, t0, dt, n_steps, L, e0_per_a0, zr_per_w0, charge / mass, dL_dr, dL_dbeta,
+    const Laser L = laser_constants(*laser);
+    TanLaser T;
+    T.kz = L.k / (2.0 * L.zR);
+    T.om_c = L.omega * kInvC0;
+    T.inv_s2c = kInvC0 / (L.sigma * L.sigma);
+    T.e0_per_a0 = kMe * kC0 * L.omega / kQe;
+    T.two_over_w0 = 2.0 / L.w0;
+    const int blocks = (int)((n_e + 31) / 32);
+    push_tangent_kernel<<<blocks, kTanThreads, 0, as_stream(stream)>>>(
+        r0, u0, n_e, t0, dt, n_steps, beam_constants(L), T, charge / mass, dL_dr, dL_dbeta,
         dL_dbeta_dot, dL_du0, dL_dlaser);
     return launch_status();
 }

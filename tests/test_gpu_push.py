@@ -1,5 +1,6 @@
-"""GPU Boris push at the edges of its electron groups (32 per CTA) and step counts, against the
-numpy pusher of the workloads, and split into blocks against one call."""
+"""GPU Boris push and its gradient at the edges of their electron groups (32 per CTA) and step
+counts: the push against the numpy pusher of the workloads, and split into blocks against one
+call; the gradient against torch autograd through the torch-written pusher."""
 import numpy as np
 import pytest
 
@@ -62,3 +63,28 @@ def test_push_in_blocks_is_bit_identical(n_e, cuts):
         for a, b in zip((R, B, A), whole[1:]):
             assert torch.equal(a, b[:, lo:hi + 1])
         lo = hi
+
+
+@pytest.mark.parametrize("n_e", [1, 32, 33])
+@pytest.mark.parametrize("n_s", [1, 2, 3, 40])
+def test_push_gradient_matches_autograd(n_e, n_s):
+    from paper_2206_03015_gb300.autograd import boris_push
+    r0, u0, t0, dt = _start(n_e, n_s)
+    g = torch.Generator().manual_seed(n_e * 100 + n_s)
+    r = torch.from_numpy(r0)
+    u = torch.from_numpy(u0).requires_grad_(True)
+    a0 = torch.tensor(LASER.a0, dtype=torch.float64, requires_grad=True)
+    w0 = torch.tensor(LASER.w0, dtype=torch.float64, requires_grad=True)
+    t, R, B, A = boris_push(r, u, a0, w0, LASER.lam, LASER.fwhm, t0, t0 + n_s * dt, n_s)
+    # every sample's position, velocity and acceleration weighted alike
+    W = [torch.randn(x.shape, dtype=torch.float64, generator=g) / float(x.detach().abs().max())
+         for x in (R, B, A)]
+    sum((w * x).sum() for w, x in zip(W, (R, B, A))).backward()
+    du, dl = lw.lw_boris_push_grad(r.cuda(), u.detach().cuda(), t0, dt, n_s, L,
+                                   *[w.cuda() for w in W])
+    # both are FP64 chains of n_s steps; the laser phase (1e3 rad) carries 1e-13 of rounding
+    # into terms that are summed with either sign
+    for got, ref in ((du.cpu(), u.grad), (dl.cpu(), torch.stack([a0.grad, w0.grad]))):
+        for c in range(got.shape[-1]):
+            a, b = got[..., c], ref[..., c]
+            assert float((a - b).norm()) <= 1e-10 * float(b.norm()), (c, a, b)
