@@ -7,11 +7,14 @@
 // z = a + i b; with Z = FFT(z):
 //   A(l) = (Z_l + conj Z_{N-l}) / 2,   B(l) = (Z_l - conj Z_{N-l}) / (2i).
 // A pixel pair (m0, m1) gives three sequences: (x0 + i y0), (x1 + i y1),
-// (z0 + i z1).  Transforms run in shared memory as passes of up to four radix-2
-// stages (lw_fft.cuh: each group pre-multiplied by twiddles from a table
-// e^{+2 pi i t/N} built once per call, then constant-root stages):
-//   N <= 4096   one CTA per pixel pair, all three sequences in turn;
-//   N >  4096   four-step: N = N1 * N2, pass 1 transforms the N2 columns of
+// (z0 + i z1).  Three forms by length (run_spectrum has the rule):
+//   N < 1024    one CTA per pixel pair, all three sequences in turn, in shared memory as
+//               passes of up to four radix-2 stages (lw_fft.cuh: each group
+//               pre-multiplied by twiddles from a table e^{+2 pi i t/N} built once
+//               per call, then constant-root stages);
+//   N <= 16384  one CTA per pixel pair, 16 elements per thread in registers, passes of
+//               radix 16 that exchange through shared memory (FP64 up to 4,096);
+//   otherwise   four-step on the passes of lw_fft.cuh: N = N1 * N2, pass 1 transforms the N2 columns of
 //               length N1 (coalesced column tiles) and applies the twiddles
 //               e^{2 pi i j2 l1 / N}, pass 2 transforms rows l1 .. l1+3 together
 //               with their mirror rows N1 - l1, which hold the Z_{N-l} needed by
@@ -155,6 +158,211 @@ __global__ void spectrum_direct_kernel(RecReader<T> rd, int64_t n_pix, int N, in
         }
         __syncthreads();
     }
+}
+
+// ---------------------------------------------------------------- one CTA, registers
+//
+// 2^10 <= N <= 2^14 (FP64: 2^12): a CTA of N/16 threads transforms a pixel pair's three
+// sequences in turn, 16 elements per thread in registers, in passes of radix 16 (the last one
+// shorter) in Stockham order: pass with Ns points already combined takes elements
+// t + i N/R of the buffer (i = 0 .. R-1), multiplies them by exp(2 pi i (t mod Ns) i/(Ns R)) and
+// stores output r of its R-point transform at (t / Ns) Ns R + t mod Ns + r Ns, so that input and
+// output are in natural order and no pass sorts.  One padding slot per 16 elements makes every
+// store and load of a half warp conflict-free.  The record is read once, coalesced, and the
+// spectrum written once: no intermediate in device memory and no zeroing.
+// Bound: shared-memory traffic (four passes over the buffer per sequence) beside the FP32 or
+// FP64 pipe.  Against the transform of one sequence at a time with run-time pass plans that this
+// replaced (up to 4,096 bins) and the four-step form (above): 2,048 pixels x 4,096 bins, FP64
+// record in FP32 arithmetic, 373 -> 68 us (3.2 TB/s of record and spectrum); FP32 record 346 ->
+// 56 us; 16,384 bins, interleaved FP32 record, 477 -> 296 us; FP64 4,096 bins 1,240 -> 1,194 us
+// (FP64 pipe).
+// Twiddles of pass (Ns, R): entry [m - 1][q] = exp(2 pi i q m/(Ns R)), q < Ns, one table per
+// pass, R = 16 passes first; N - 16 entries in all.
+template <typename T>
+__global__ void pass_twiddle_kernel(typename V2<T>::type* tw, int logN) {
+    const int n = (1 << logN) - 16;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+        int off = 0, logNs = 4;
+        while (true) {   // the pass that holds entry e
+            const int logR = min(4, logN - logNs);
+            const int cnt = ((1 << logR) - 1) << logNs;
+            if (e < off + cnt) break;
+            off += cnt;
+            logNs += logR;
+        }
+        const int logR = min(4, logN - logNs);
+        const int m = ((e - off) >> logNs) + 1, q = (e - off) & ((1 << logNs) - 1);
+        double s, c;
+        sincospi(2.0 * (double)(q * m) / (double)(1 << (logNs + logR)), &s, &c);
+        typename V2<T>::type w;
+        w.x = (T)c;
+        w.y = (T)s;
+        tw[e] = w;
+    }
+}
+
+// R-point transform (sign +) in registers; output k is left in x[rev(k)].
+template <typename C, int R>
+__device__ __forceinline__ void fft_regs(C* x) {
+#pragma unroll
+    for (int half = R / 2; half >= 1; half >>= 1) {
+#pragma unroll
+        for (int m = 0; m < R; ++m) {
+            if (m & half) continue;
+            const C u = x[m], v = x[m + half];
+            x[m] = cadd(u, v);
+            x[m + half] = mul_root16(csub(u, v), (m & (half - 1)) * (8 / half));
+        }
+    }
+}
+
+template <int LOGN>
+struct RegPlan {
+    static constexpr int N = 1 << LOGN, T = N / 16;
+    static constexpr int slots = N + N / 16;
+    // resident CTAs that the register limit leaves room for: FP32 80 registers a thread (64 with
+    // 2^13 and 2^14 points, where a CTA is 512 or 1,024 threads), FP64 128
+    template <typename U> static constexpr int min_ctas() {
+        return sizeof(U) == 8 ? 512 / T : LOGN <= 12 ? 768 / T : 1024 / T;
+    }
+};
+__device__ __forceinline__ int reg_slot(int j) { return j + (j >> 4); }
+
+// Passes from LOGNS on over v (in: element t + i N/16 of the pass's input is v[i]); the last
+// pass's output stays in v with element index tb + r N/R at v[b R + rev(r)].
+template <typename C, int LOGN, int LOGNS>
+__device__ __forceinline__ void reg_passes(C* v, C* buf, const C* __restrict__ tw) {
+    constexpr int N = 1 << LOGN, T = N / 16;
+    constexpr int LOGR = LOGN - LOGNS < 4 ? LOGN - LOGNS : 4, R = 1 << LOGR, M = 16 / R;
+    constexpr int Ns = 1 << LOGNS;
+    const int t = threadIdx.x;
+    // v[i] holds element t + i T; butterfly b of the thread takes elements (t + b T) + i N/R,
+    // i.e. v[b + i M]
+    C x[16];
+#pragma unroll
+    for (int b = 0; b < M; ++b) {
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            x[b * R + i] = v[b + i * M];
+            if (LOGNS > 0 && i > 0) {
+                const int q = (t + b * T) & (Ns - 1);
+                x[b * R + i] = cmul(x[b * R + i], tw[(i - 1) * Ns + q]);
+            }
+        }
+        fft_regs<C, R>(x + b * R);
+    }
+    if constexpr (LOGNS + LOGR < LOGN) {
+        if (LOGNS > 0) __syncthreads();   // the pass before has read its elements
+#pragma unroll
+        for (int b = 0; b < M; ++b) {
+            const int tb = t + b * T;
+            const int d = ((tb >> LOGNS) << (LOGNS + LOGR)) + (tb & (Ns - 1));
+#pragma unroll
+            for (int r = 0; r < R; ++r) buf[reg_slot(d + r * Ns)] = x[b * R + rev_bits(r, LOGR)];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = buf[reg_slot(t + i * T)];
+        reg_passes<C, LOGN, LOGNS + LOGR>(v, buf, tw + (LOGNS > 0 ? (R - 1) * Ns : 0));
+    } else {
+        __syncthreads();
+#pragma unroll
+        for (int b = 0; b < M; ++b)
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                buf[reg_slot(t + b * T + r * (N / R))] = x[b * R + rev_bits(r, LOGR)];
+        __syncthreads();
+    }
+}
+
+template <typename T, int LOGN>
+__global__ void __launch_bounds__(RegPlan<LOGN>::T, RegPlan<LOGN>::template min_ctas<T>())
+    spectrum_regs_kernel(RecReader<T> rd, int64_t n_pix, T scale,
+                         const typename V2<T>::type* __restrict__ tw, T* __restrict__ S,
+                         typename V2<T>::type* __restrict__ X) {
+    using C = typename V2<T>::type;
+    using Raw = typename RecReader<T>::Raw;
+    constexpr int N = 1 << LOGN, TH = N / 16;
+    constexpr int64_t nl = N / 2 + 1;
+    extern __shared__ unsigned char smem_raw[];
+    C* buf = reinterpret_cast<C*>(smem_raw);
+    const int t = threadIdx.x;
+    const int64_t pair = blockIdx.x;
+    // sequences in the order (x0, y0), (z0, z1), (x1, y1), so that one pixel's partial powers
+    // are kept at a time: thread t's are at l = t + q N/16, and l = N/2 with thread 0
+    T acc[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) acc[q] = (T)0;
+#pragma unroll 1
+    for (int step = 0; step < 3; ++step) {
+        const int kind = step == 0 ? 0 : 3 - step;
+        const SeqRows sr = seq_rows(pair, kind, n_pix);
+        if (sr.ma < 0) continue;   // uniform: no second pixel
+        C v[16];
+        {
+            constexpr int kBatch = sizeof(Raw) == 8 && sizeof(T) == 4 ? 8 : 16;
+#pragma unroll
+            for (int i0 = 0; i0 < 16; i0 += kBatch) {
+                Raw va[kBatch], vb[kBatch];
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) {
+                    const int j = t + (i0 + u) * TH;
+                    va[u] = rd.load(sr.ra, N, j);
+                    vb[u] = sr.rb >= 0 ? rd.load(sr.rb, N, j) : Raw{};
+                }
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) {
+                    v[i0 + u].x = (scale * rd.cvt_fp64(va[u])) * scale;
+                    v[i0 + u].y = (scale * rd.cvt(vb[u])) * scale;
+                }
+            }
+        }
+        reg_passes<C, LOGN, 0>(v, buf, tw);
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            const int l = t + q * TH;
+            if (q == 8 && t != 0) break;
+            const C zl = buf[reg_slot(l)], zn = buf[reg_slot((N - l) & (N - 1))];
+            // s = zl + zn, d = zl - zn: the two rows' spectra are A = (s.x, d.y) / 2 and
+            // B = (s.y, -d.x) / 2
+            const C sv = cadd(zl, zn), dv = csub(zl, zn);
+            C A, B;
+            A.x = (T)0.5 * sv.x;
+            A.y = (T)0.5 * dv.y;
+            B.x = (T)0.5 * sv.y;
+            B.y = (T)-0.5 * dv.x;
+            const T pa = A.x * A.x + A.y * A.y, pb = B.x * B.x + B.y * B.y;
+            if (X) {
+                X[(sr.ma * 3 + sr.ca) * nl + l] = A;
+                if (sr.mb >= 0) X[(sr.mb * 3 + sr.cb) * nl + l] = B;
+            }
+            if (kind == 0) {
+                acc[q] = pa + pb;
+            } else if (kind == 2) {   // pixel 0 is complete; pixel 1 (if any) starts
+                S[sr.ma * nl + l] = acc[q] + pa;
+                acc[q] = pb;
+            } else {
+                S[sr.ma * nl + l] = acc[q] + (pa + pb);
+            }
+        }
+        __syncthreads();   // the buffer is rewritten by the next sequence
+    }
+}
+
+template <typename T, int LOGN>
+int launch_regs(const RecReader<T>& rd, int64_t n_pix, T scale, typename V2<T>::type* tw, T* S,
+                typename V2<T>::type* X, cudaStream_t st) {
+    using C = typename V2<T>::type;
+    const int64_t pairs = (n_pix + 1) / 2;
+    const size_t smem = sizeof(C) * (size_t)RegPlan<LOGN>::slots;
+    const auto kern = spectrum_regs_kernel<T, LOGN>;
+    if (smem > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)smem) != cudaSuccess)
+        return LW_ECUDA;
+    pass_twiddle_kernel<T><<<(RegPlan<LOGN>::N + 127) / 128, 128, 0, st>>>(tw, LOGN);
+    if (launch_status() != LW_OK) return LW_ECUDA;
+    kern<<<(unsigned)pairs, RegPlan<LOGN>::T, smem, st>>>(rd, n_pix, scale, tw, S, X);
+    return launch_status();
 }
 
 // ---------------------------------------------------------------- four-step
@@ -371,6 +579,13 @@ int run_spectrum(const void* record, int kind, int64_t n_pix, const lw_grid* g, 
     const int64_t N = g->n_bins;
     int logN = 0;
     while ((int64_t(1) << logN) < N) ++logN;
+    // one CTA per pixel pair where a pair's sequence fits and, above 4,096 bins, where the
+    // pairs fill half of the SMs (a CTA is then 512 or 1,024 threads).  Interleaved FP32
+    // records, one CTA per pair against four-step: 2,048 pixels x 16,384 bins 296 and 477 us,
+    // 400 pixels 81 and 107, 200 pixels 42 and 59, 100 pixels 40 and 37; 8,192 bins and 200
+    // pixels 37 and 37, 400 pixels 39 and 57.  FP64 at 8,192 bins: 400 pixels 742 and 579.
+    const bool regs = N >= 1024 && (N <= 4096 || (sizeof(T) == 4 && N <= 16384 &&
+                                                  (n_pix + 1) / 2 >= kSms / 2));
     const bool direct = N <= 4096;
     const int64_t n_pairs = (n_pix + 1) / 2;
     const int64_t n_seq = 3 * n_pairs;
@@ -397,6 +612,17 @@ int run_spectrum(const void* record, int kind, int64_t n_pix, const lw_grid* g, 
     C* X = static_cast<C*>(X_save);
     const int nl = (int)(N / 2 + 1);
 
+    if (regs) {
+        switch (logN) {
+            case 10: return launch_regs<T, 10>(rd, n_pix, scale, tw, S, X, st);
+            case 11: return launch_regs<T, 11>(rd, n_pix, scale, tw, S, X, st);
+            case 12: return launch_regs<T, 12>(rd, n_pix, scale, tw, S, X, st);
+            default:
+                if constexpr (sizeof(T) == 4)
+                    return logN == 13 ? launch_regs<T, 13>(rd, n_pix, scale, tw, S, X, st)
+                                      : launch_regs<T, 14>(rd, n_pix, scale, tw, S, X, st);
+        }
+    }
     const int tw_grid = (int)((N + 255) / 256 < 1024 ? (N + 255) / 256 : 1024);
     twiddle_kernel<T><<<tw_grid, 256, 0, st>>>(tw, N);
     if (launch_status() != LW_OK) return LW_ECUDA;
