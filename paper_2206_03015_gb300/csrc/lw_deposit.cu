@@ -9,12 +9,11 @@
 // contributions are added to the record with global atomics (pixels of
 // different CTAs share bins through electrons of other chunks).
 //
-// FP64 path: every step costs the time map and one compare.  Every operation
-// of the time map, the bin index, the field and the weights is written with
-// explicit round-to-nearest intrinsics in the order documented in lw.h, so
-// advanced times, bin indices and per-sample contributions are bit-identical
-// to a plain C loop without FMA contraction; only the order of the atomic
-// additions differs.
+// FP64 path (deposit_fp64_kernel): every result of the time map, the bin index,
+// the field and the weights is the correctly rounded one of the operation order
+// documented in lw.h, so advanced times, bin indices and per-sample contributions
+// are bit-identical to a plain C loop without FMA contraction; only the order of
+// the atomic additions differs.
 //
 // Mixed path: the bin coordinate u = (t_a - t_min)/dt_u is anchored once per
 // block of samples in double-FP32 arithmetic (integer part + FP32 fraction)
@@ -73,18 +72,52 @@ struct DepositArgs {
 constexpr int kFp64Threads = 128;
 constexpr int kFp64Tile = 64;
 
+// FP64 instructions are what these kernels pay for (GB300: 19 cycles per warp instruction and
+// SM), so quotients with a common divisor share its correctly rounded reciprocal r: with one
+// residual correction n r is the correctly rounded quotient (Markstein), 3 instructions after
+// the 5 of the reciprocal instead of 8 per division.  Where the product or the correction
+// leaves the finite range the division itself decides
+// (a call, so that its instructions are not issued beside the common path under a predicate).
+__device__ __noinline__ double divide_rare(double n, double d) { return __ddiv_rn(n, d); }
+__device__ __forceinline__ double quotient(double n, double d, double r) {
+    double q = __dmul_rn(n, r);
+    q = __fma_rn(__fma_rn(-q, d, n), r, q);
+    if ((__double2hiint(q) & 0x7ff00000) == 0x7ff00000) q = divide_rare(n, d);
+    return q;
+}
+// x > 0 and |x| < 2^62 on the bits (integer pipe; NaN and infinities fail)
+__device__ __forceinline__ bool positive(double x) {
+    const int hi = __double2hiint(x);
+    return hi > 0 && hi < 0x7ff00000;
+}
+__device__ __forceinline__ bool in_range(double u) {
+    return (__double2hiint(u) & 0x7fffffff) < 0x43d00000;
+}
+
+// |beta|^2 < 1, decided in FP32 where 1 - beta^2 is far above its FP32 rounding (as in the
+// upload), else by the FP64 expression ((bx*bx + by*by) + bz*bz) < 1
+__device__ __noinline__ bool subluminal_exact(double b0, double b1, double b2) {
+    return __dadd_rn(__dadd_rn(__dmul_rn(b0, b0), __dmul_rn(b1, b1)), __dmul_rn(b2, b2)) < 1.0;
+}
+__device__ __forceinline__ bool subluminal(double b0, double b1, double b2) {
+    const float eps = to_float(1.0 - b2);
+    const float x = to_float(b0), y = to_float(b1);
+    const float perp = fmaf(x, x, y * y);
+    const float one_minus = fmaf(-eps, eps, 2.0f * eps) - perp;
+    if (__double2hiint(b2) >= 0x3fe00000 && one_minus > 1.0e-5f * (2.0f * eps + perp)) return true;
+    return subluminal_exact(b0, b1, b2);
+}
+
 // Field of one sample with the oracle's operation order (see lw.h).
 __device__ int field_fp64(double nx, double ny, double nz, double R, uint32_t flags,
                           const double* __restrict__ b, const double* __restrict__ a,
                           double F[3]) {
     F[0] = F[1] = F[2] = 0.0;
     const double b0 = b[0], b1 = b[1], b2v = b[2];
-    const double bb = __dadd_rn(__dadd_rn(__dmul_rn(b0, b0), __dmul_rn(b1, b1)),
-                                __dmul_rn(b2v, b2v));
     const double nb = __dadd_rn(__dadd_rn(__dmul_rn(nx, b0), __dmul_rn(ny, b1)),
                                 __dmul_rn(nz, b2v));
     const double D = __dsub_rn(1.0, nb);
-    if (!(bb < 1.0) || !(D > 0.0)) return LW_ST_BETA;
+    if (!positive(D) || !subluminal(b0, b1, b2v)) return LW_ST_BETA;
     const double D3 = __dmul_rn(__dmul_rn(D, D), D);
     const double m0 = __dsub_rn(nx, b0), m1 = __dsub_rn(ny, b1), m2 = __dsub_rn(nz, b2v);
     if (flags & LW_FIELD_ACCEL) {
@@ -97,17 +130,32 @@ __device__ int field_fp64(double nx, double ny, double nz, double R, uint32_t fl
         const double o0 = __dsub_rn(__dmul_rn(ny, i2), __dmul_rn(nz, i1));
         const double o1 = __dsub_rn(__dmul_rn(nz, i0), __dmul_rn(nx, i2));
         const double o2 = __dsub_rn(__dmul_rn(nx, i1), __dmul_rn(ny, i0));
-        F[0] = __ddiv_rn(o0, D3);
-        F[1] = __ddiv_rn(o1, D3);
-        F[2] = __ddiv_rn(o2, D3);
+        const double r = __drcp_rn(D3);
+        F[0] = quotient(o0, D3, r);
+        F[1] = quotient(o1, D3, r);
+        F[2] = quotient(o2, D3, r);
     }
     if (flags & LW_FIELD_VELOCITY) {
+        const double bb = __dadd_rn(__dadd_rn(__dmul_rn(b0, b0), __dmul_rn(b1, b1)),
+                                    __dmul_rn(b2v, b2v));
         const double g = __ddiv_rn(__dmul_rn(kC0, __dsub_rn(1.0, bb)), __dmul_rn(D3, R));
         F[0] = __dadd_rn(F[0], __dmul_rn(m0, g));
         F[1] = __dadd_rn(F[1], __dmul_rn(m1, g));
         F[2] = __dadd_rn(F[2], __dmul_rn(m2, g));
     }
     return 0;
+}
+
+// The interpolated value of Algorithm 2 at grid point j (as a double) of the step (tb, ta] with
+// the fields Fb, Fa at its ends and r = 1/(ta - tb), added to the pixel's rows at rec.
+__device__ __forceinline__ void deposit_fp64(const DepositArgs& p, double* rec, double j, double ta,
+                                             double tb, double den, double r, const double Fa[3],
+                                             const double Fb[3]) {
+    const double tu = __dadd_rn(p.t_min, __dmul_rn(j, p.dt_u));
+    const double wa = quotient(__dsub_rn(ta, tu), den, r);
+    const double wb = quotient(__dsub_rn(tu, tb), den, r);
+    for (int c = 0; c < 3; ++c)
+        atomicAdd(rec + c * p.n_bins, __dadd_rn(__dmul_rn(Fb[c], wa), __dmul_rn(Fa[c], wb)));
 }
 
 // State of Algorithm 2's walk over one (pixel, electron): the previous sample's
@@ -133,13 +181,13 @@ __device__ __forceinline__ void scan_sample(const DepositArgs& p, double nx, dou
                                             double y, double z, ScanState& S, int& bits) {
     const double ta = advanced_time_fp64(nx, ny, nz, x, y, z, t);
     const double ua = __dmul_rn(__dsub_rn(ta, p.t_min), p.inv_dtu);
-    const bool ok_a = fabs(ua) < 4.0e18;
+    const bool ok_a = in_range(ua);
     if (i > 0) {
         if (!ok_a || !S.ok_b) {
             bits |= LW_ST_NONFINITE;
         } else {
-            const int64_t j_hi = (int64_t)floor(ua);
-            const int64_t j_lo = (int64_t)floor(S.ub) + 1;
+            const int64_t j_hi = __double2ll_rd(ua);
+            const int64_t j_lo = __double2ll_rd(S.ub) + 1;
             if (!(ta > S.tb)) bits |= LW_ST_TA_ORDER;
             if (j_lo <= j_hi) {
                 int64_t ja = j_lo, jz = j_hi;
@@ -158,14 +206,10 @@ __device__ __forceinline__ void scan_sample(const DepositArgs& p, double nx, dou
                     double Fa[3];
                     field_fp64(nx, ny, nz, p.R, p.flags, bk + 3 * i, ak + 3 * i, Fa);
                     const double den = __dsub_rn(ta, S.tb);
-                    for (int64_t j = ja; j <= jz; ++j) {
-                        const double tu = __dadd_rn(p.t_min, __dmul_rn((double)j, p.dt_u));
-                        const double wa = __ddiv_rn(__dsub_rn(ta, tu), den);
-                        const double wb = __ddiv_rn(__dsub_rn(tu, S.tb), den);
-                        for (int c = 0; c < 3; ++c)
-                            atomicAdd(rec + c * p.n_bins + j,
-                                      __dadd_rn(__dmul_rn(S.Fb[c], wa), __dmul_rn(Fa[c], wb)));
-                    }
+                    const double r = __drcp_rn(den);
+                    double jd = (double)ja;
+                    for (int64_t j = ja; j <= jz; ++j, jd += 1.0)
+                        deposit_fp64(p, rec + j, jd, ta, S.tb, den, r, Fa, S.Fb);
                     S.Fb[0] = Fa[0];
                     S.Fb[1] = Fa[1];
                     S.Fb[2] = Fa[2];
@@ -1002,40 +1046,45 @@ __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int
     return bits;
 }
 
-// FP64 deposit for trajectories whose advanced time increases (no LW_ST_STEP
-// from the upload): per pixel and block of samples, the grid points reached
-// are the run (floor(u_b), floor(u_end)]; each is located, by a bracketed
-// search over the staged block, at the first sample whose coordinate reaches
-// it -- the step of Algorithm 2 that holds it -- and deposited with the scan's
-// FP64 expressions in the oracle's operation order, so every contribution is
-// bit-identical to the literal scan (only the order of the atomic additions
-// differs).  With LW_ST_STEP set the literal scan runs instead, and electrons that
-// reach more than half a grid point per step (on average over the CTA's pixels) are
-// walked step by step, like the scan, from the same staged blocks.
-constexpr int kF64Block = 256;   // samples staged per block
+// FP64 deposit, CTA = 128 pixels x one electron (x a part of it, grid z), every contribution
+// bit-identical to the literal scan (only the order of the atomic additions differs).  What
+// bounds it is the FP64 pipe, so the work is arranged to keep every lane of an FP64 instruction
+// busy, in one of two forms chosen per electron by the CTA:
+//  * few grid points per step (trajectories whose advanced time increases): a pixel's grid
+//    points are the run (floor(u_first), floor(u_last)] of the whole trajectory.  The CTA's
+//    runs are listed by a prefix sum and taken one grid point per thread; a thread searches its
+//    grid point's step among the stored samples (interpolation, then bisection) with the
+//    difference u - j in three FP64 instructions and FP32, confirms the two samples with
+//    the scan's coordinate and deposits.  Samples are read where the search lands, nothing is
+//    staged.  (A search per staged block of 256 samples left 5 of 32 lanes busy at 3 grid
+//    points per trajectory: 1,000 electrons x 5,000 steps x 1,024 pixels 7.9 ms, now 1.3 ms.)
+//  * more than half a grid point per step on average: every step in order from staged blocks,
+//    fields once per step (64 electrons x 1,200 steps x 400 pixels x 4,096 bins, 3.4 points
+//    per step: 17.0 ms before the shared reciprocals and the division over grid z, now 9.0).
+// Inputs that the upload flagged (a step longer than c0 dt, times out of order, non-finite
+// values) take the literal scan.
+constexpr int kF64Block = 64;   // samples staged per block
 
-__global__ void __launch_bounds__(kFp64Threads) deposit_fp64_jobs_kernel(DepositArgs p) {
-    if (p.input_status && (*p.input_status & LW_ST_STEP)) {
-        fp64_scan_cta(p);
+__global__ void __launch_bounds__(kFp64Threads) deposit_fp64_kernel(DepositArgs p) {
+    if (p.input_status && (*p.input_status & (LW_ST_STEP | LW_ST_TIME | LW_ST_NONFINITE))) {
+        if (blockIdx.z == 0) fp64_scan_cta(p);
         return;
     }
-    constexpr int kWarpsF = kFp64Threads / 32;
     __shared__ double s_t[2][kF64Block + 1];        // sample i0-1 first
     __shared__ double s_r[2][3 * (kF64Block + 1)];
     __shared__ double s_n[kFp64Threads][3];         // pixel directions
-    __shared__ double s_ua[kFp64Threads];           // block: coordinate before the block
-    __shared__ double s_ue[kFp64Threads];           // block: coordinate of its last sample
-    __shared__ int s_ja[kFp64Threads];              // block: first grid point of the run
-    __shared__ int s_kp[kFp64Threads];              // block: job offset in the warp
-    __shared__ int2 s_tab[kWarpsF][kJobTable];      // block: (slot, grid point) of job t
-    __shared__ unsigned long long s_pts[2];         // grid points of the electron (alternating)
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int wslot = warp * 32;
+    __shared__ float s_w[kFp64Threads][3];          // and slopes
+    __shared__ double s_u[kFp64Threads][2];         // coordinates of the first and last sample
+    __shared__ int s_ja[kFp64Threads];              // first grid point of the run
+    __shared__ long long s_off[kFp64Threads];       // grid points of the pixels before
+    __shared__ long long s_warp[kFp64Threads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t pix0 = (int64_t)blockIdx.x * kFp64Threads;
     const int n_act = (int)min((int64_t)kFp64Threads, p.n_pix - pix0);
     const int64_t m = pix0 + threadIdx.x;
     const bool active = m < p.n_pix;
     const int nb = (int)p.n_bins;
+    const int last = (int)(p.ns1 - 1);
     double nx = 0.0, ny = 0.0, nz = 1.0;
     if (active) {
         nx = p.n_hat[3 * m];
@@ -1045,197 +1094,156 @@ __global__ void __launch_bounds__(kFp64Threads) deposit_fp64_jobs_kernel(Deposit
     s_n[threadIdx.x][0] = nx;
     s_n[threadIdx.x][1] = ny;
     s_n[threadIdx.x][2] = nz;
+    {   // slopes of u with the transverse position and with z beside tau, in FP32
+        const double sc = kInvC0 * p.inv_dtu;
+        s_w[threadIdx.x][0] = to_float(-nx * sc);
+        s_w[threadIdx.x][1] = to_float(-ny * sc);
+        s_w[threadIdx.x][2] = to_float((1.0 - nz) * sc);
+    }
     int bits = 0;
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && p.input_status)
+    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0 &&
+        p.input_status)
         bits |= *p.input_status;
     const int nblk = (int)((p.ns1 + kF64Block - 1) / kF64Block);
-    auto electron = [&](int64_t kk) -> int64_t { return p.order ? (int64_t)p.order[kk] : kk; };
-    auto issue = [&](int64_t k, int b, int buf) {
-        const int64_t i0 = (int64_t)b * kF64Block;
-        const int n = (int)min((int64_t)kF64Block, p.ns1 - i0);
-        const double* tk = p.t + (p.t_per_e ? k * p.ns1 : 0) + i0;
-        const double* rk = p.r + 3 * (k * p.ns1 + i0);
-        for (int q = (b == 0 ? 1 : 0) + threadIdx.x; q <= n; q += kFp64Threads)
-            cp_async8(&s_t[buf][q], tk + (q - 1));
-        for (int q = (b == 0 ? 3 : 0) + threadIdx.x; q < 3 * (n + 1); q += kFp64Threads)
-            cp_async8(&s_r[buf][q], rk + (q - 3));
-        cp_async_commit();
-    };
-    // coordinate u = (t_a - t_min) / dt_u of staged sample q, the scan's expression
-    auto coord64 = [&](const double* n3, int buf, int q) -> double {
-        const double ta = advanced_time_fp64(n3[0], n3[1], n3[2], s_r[buf][3 * q],
-                                             s_r[buf][3 * q + 1], s_r[buf][3 * q + 2],
-                                             s_t[buf][q]);
-        return __dmul_rn(__dsub_rn(ta, p.t_min), p.inv_dtu);
-    };
+    auto coord = [&](double ta) { return __dmul_rn(__dsub_rn(ta, p.t_min), p.inv_dtu); };
     const int64_t k0 = (int64_t)blockIdx.y * p.e_chunk;
     const int64_t k1 = min(k0 + p.e_chunk, p.n_e);
-    int buf = 0;
-    if (k0 < k1) issue(electron(k0), 0, 0);
     for (int64_t kk = k0; kk < k1; ++kk) {
-        const int64_t k = electron(kk);
+        const int64_t k = p.order ? (int64_t)p.order[kk] : kk;
+        const double* tk = p.t + (p.t_per_e ? k * p.ns1 : 0);
+        const double* rk = p.r + 3 * k * p.ns1;
         const double* bk = p.beta + 3 * k * p.ns1;
         const double* ak = p.bdot + 3 * k * p.ns1;
         const double* e0 = p.ends + 8 * k;
-        const double u0 = __dmul_rn(__dsub_rn(advanced_time_fp64(nx, ny, nz, e0[1], e0[2], e0[3],
-                                                                 e0[0]),
-                                              p.t_min),
-                                    p.inv_dtu);
-        bool ok = fabs(u0) < 4.0e18;
-        if (active && !ok) bits |= LW_ST_NONFINITE;
-        int64_t jdone = ok ? (int64_t)floor(u0) : 0;
-        double uprev = u0;
-        // More than half a grid point per step on average over the CTA's pixels: walk
-        // every step (fields once per step, shared by the grid points it holds) instead
-        // of locating each grid point -- the choice is the CTA's, per electron.
-        const double ul = __dmul_rn(__dsub_rn(advanced_time_fp64(nx, ny, nz, e0[5], e0[6], e0[7],
-                                                                 e0[4]),
-                                              p.t_min),
-                                    p.inv_dtu);
-        unsigned long long pts = 0;
-        if (active && ok && fabs(ul) < 4.0e18) {
-            const double lo = fmax(floor(u0), -1.0), hi = fmin(floor(ul), (double)nb - 1.0);
-            if (hi > lo) pts = (unsigned long long)(hi - lo);
+        const double u0 = coord(advanced_time_fp64(nx, ny, nz, e0[1], e0[2], e0[3], e0[0]));
+        const double ul = coord(advanced_time_fp64(nx, ny, nz, e0[5], e0[6], e0[7], e0[4]));
+        const bool ok = in_range(u0) && in_range(ul);
+        int64_t a = 0, z = -1;   // the pixel's run
+        if (active && ok) {
+            a = __double2ll_rd(u0) + 1;
+            z = __double2ll_rd(ul);
         }
-        for (int o = 16; o > 0; o >>= 1) pts += __shfl_down_sync(0xffffffffu, pts, o);
-        const int ci = (int)(kk & 1);
-        if (threadIdx.x == 0) s_pts[ci] = 0;
-        __syncthreads();
-        if (lane == 0) atomicAdd(&s_pts[ci], pts);
-        __syncthreads();
-        const bool per_step = 2 * s_pts[ci] > (unsigned long long)n_act * (unsigned long long)(p.ns1 - 1);
-        ScanState S;
-        S.reset();
-        double* rec_m = static_cast<double*>(p.record) + (active ? m * 3 * p.n_bins : 0);
-        for (int b = 0; b < nblk; ++b) {
-            const int64_t i0 = (int64_t)b * kF64Block;
-            const int n = (int)min((int64_t)kF64Block, p.ns1 - i0);
-            cp_async_wait_all();
-            __syncthreads();   // block b staged; every warp is done with block b-1
-            if (b + 1 < nblk)
-                issue(k, b + 1, buf ^ 1);
-            else if (kk + 1 < k1)
-                issue(electron(kk + 1), 0, buf ^ 1);
-            const int cb = buf;
-            buf ^= 1;
-            if (per_step) {
-                if (active)
-                    for (int q = 1; q <= n; ++q)
-                        scan_sample(p, nx, ny, nz, rec_m, bk, ak, i0 + q - 1, s_t[cb][q],
-                                    s_r[cb][3 * q], s_r[cb][3 * q + 1], s_r[cb][3 * q + 2], S,
-                                    bits);
-                continue;
-            }
-            const int lo0 = (b == 0) ? 1 : 0;   // sample 0 ends no step
-            const double ue = coord64(s_n[threadIdx.x], cb, n);
-            int K = 0, ja = 0, big = 0;
-            if (active && ok && n > lo0) {
-                if (!(fabs(ue) < 4.0e18)) {
-                    bits |= LW_ST_NONFINITE;
-                    ok = false;
-                } else {
-                    const int64_t jend = (int64_t)floor(ue);
-                    int64_t a = jdone + 1, z = jend;
-                    if (a <= z) {
-                        if (a < 0) {
-                            a = 0;
-                            bits |= LW_ST_CLIP;
-                        }
-                        if (z > nb - 1) {
-                            z = nb - 1;
-                            bits |= LW_ST_CLIP;
-                        }
-                        if (a <= z) {
-                            K = (int)(z - a + 1);
-                            ja = (int)a;
-                            if (K > kMaxWarpJobs) {
-                                big = K;
-                                K = 0;
-                            }
-                        }
-                    }
-                    if (jend > jdone) jdone = jend;
-                }
-            }
-            s_ja[threadIdx.x] = ja;
-            s_ua[threadIdx.x] = b == 0 ? u0 : uprev;
-            s_ue[threadIdx.x] = ue;
-            uprev = ue;
-            // the warp's grid points: prefix sum, the first kJobTable listed by owners
-            int incl = K;
+        const bool clipped = a <= z && (a < 0 || z > nb - 1);
+        a = max(a, (int64_t)0);
+        z = min(z, (int64_t)nb - 1);
+        const int K = a <= z ? (int)(z - a + 1) : 0;
+        // prefix sum of the runs over the CTA
+        long long incl = K;
 #pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const int v = __shfl_up_sync(0xffffffffu, incl, d);
-                if (lane >= d) incl += v;
-            }
-            const int T = __shfl_sync(0xffffffffu, incl, 31);
-            const int run = incl - K;
-            s_kp[threadIdx.x] = run;
-            for (int t = 0; t < K && run + t < kJobTable; ++t)
-                s_tab[warp][run + t] = make_int2(threadIdx.x, ja + t);
-            __syncwarp();
-            // grid point j of slot sl: locate its step in the staged block and deposit
-            auto job = [&](int sl, int j) {
-                const double* n3 = s_n[sl];
-                const double J = (double)j;
-                // first staged sample in [lo0, n-1] (local index) with u >= j
-                int a = lo0 - 1, hb = n - 1;
-                double xa = s_ua[sl], xb = s_ue[sl];
-                int probes = 0;
-                while (hb - a > 1) {
-                    int g = (a + hb) >> 1;
-                    if (probes < kFalsiProbes) {
-                        const float fr = __fdividef((float)(J - xa), (float)(xb - xa));
-                        const float gf = ceilf(fr * (float)(hb - a));
-                        g = a + (int)fminf(fmaxf(gf, 1.0f), (float)(hb - a - 1));
-                    }
-                    ++probes;
-                    const double xg = coord64(n3, cb, g + 1);
-                    if (xg >= J) {
-                        hb = g;
-                        xb = xg;
-                    } else {
-                        a = g;
-                        xa = xg;
-                    }
-                }
-                const int i = hb;   // local index of the step's end sample
-                const int q = i + 1;
-                const double ta = advanced_time_fp64(n3[0], n3[1], n3[2], s_r[cb][3 * q],
-                                                     s_r[cb][3 * q + 1], s_r[cb][3 * q + 2],
-                                                     s_t[cb][q]);
-                const double tb = advanced_time_fp64(n3[0], n3[1], n3[2], s_r[cb][3 * q - 3],
-                                                     s_r[cb][3 * q - 2], s_r[cb][3 * q - 1],
-                                                     s_t[cb][q - 1]);
-                const int64_t gi = i0 + i;   // global sample index of the step's end
-                double Fb[3], Fa[3];
-                field_fp64(n3[0], n3[1], n3[2], p.R, p.flags, bk + 3 * (gi - 1), ak + 3 * (gi - 1),
-                           Fb);
-                field_fp64(n3[0], n3[1], n3[2], p.R, p.flags, bk + 3 * gi, ak + 3 * gi, Fa);
-                const double den = __dsub_rn(ta, tb);
-                const double tu = __dadd_rn(p.t_min, __dmul_rn(J, p.dt_u));
-                const double wa = __ddiv_rn(__dsub_rn(ta, tu), den);
-                const double wb = __ddiv_rn(__dsub_rn(tu, tb), den);
-                double* rec = static_cast<double*>(p.record) + (pix0 + sl) * 3 * p.n_bins + j;
-                for (int c = 0; c < 3; ++c)
-                    atomicAdd(rec + c * p.n_bins,
-                              __dadd_rn(__dmul_rn(Fb[c], wa), __dmul_rn(Fa[c], wb)));
+        for (int d = 1; d < 32; d <<= 1) {
+            const long long v = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += v;
+        }
+        __syncthreads();   // the electron before is done with the shared arrays
+        if (lane == 31) s_warp[warp] = incl;
+        s_ja[threadIdx.x] = (int)a;
+        s_u[threadIdx.x][0] = u0;
+        s_u[threadIdx.x][1] = ul;
+        const int bad = __syncthreads_or(active && !ok);
+        long long before = 0, T = 0;
+        for (int w = 0; w < kFp64Threads / 32; ++w) {
+            if (w < warp) before += s_warp[w];
+            T += s_warp[w];
+        }
+        s_off[threadIdx.x] = before + incl - K;
+        __syncthreads();
+        if (bad || 2 * T > (long long)n_act * last) {
+            // every step of the CTA's part of the blocks, in order
+            const int b0 = (int)((int64_t)nblk * blockIdx.z / gridDim.z);
+            const int b1 = (int)((int64_t)nblk * (blockIdx.z + 1) / gridDim.z);
+            auto issue = [&](int b, int buf) {
+                const int64_t i0 = (int64_t)b * kF64Block;
+                const int n = (int)min((int64_t)kF64Block, p.ns1 - i0);
+                for (int q = (b == 0 ? 1 : 0) + threadIdx.x; q <= n; q += kFp64Threads)
+                    cp_async8(&s_t[buf][q], tk + i0 + (q - 1));
+                for (int q = (b == 0 ? 3 : 0) + threadIdx.x; q < 3 * (n + 1); q += kFp64Threads)
+                    cp_async8(&s_r[buf][q], rk + 3 * i0 + (q - 3));
+                cp_async_commit();
             };
-            for (int t = lane; t < T; t += 32) {
-                if (t < kJobTable) {
-                    const int2 e = s_tab[warp][t];
-                    job(e.x, e.y);
-                } else {
-                    int pos = 0;
+            ScanState S;
+            S.reset();
+            double* rec_m = static_cast<double*>(p.record) + (active ? m * 3 * p.n_bins : 0);
+            if (b0 < b1) issue(b0, 0);
+            for (int b = b0; b < b1; ++b) {
+                const int64_t i0 = (int64_t)b * kF64Block;
+                const int n = (int)min((int64_t)kF64Block, p.ns1 - i0);
+                const int cb = (b - b0) & 1;
+                cp_async_wait_all();
+                __syncthreads();   // block b staged; every warp is done with block b-1
+                if (b + 1 < b1) issue(b + 1, cb ^ 1);
+                if (!active) continue;
+                if (b == b0 && b > 0) {   // the sample before the first block
+                    S.tb = advanced_time_fp64(nx, ny, nz, s_r[cb][0], s_r[cb][1], s_r[cb][2],
+                                              s_t[cb][0]);
+                    S.ub = coord(S.tb);
+                    S.ok_b = in_range(S.ub);
+                }
+                for (int q = 1; q <= n; ++q)
+                    scan_sample(p, nx, ny, nz, rec_m, bk, ak, i0 + q - 1, s_t[cb][q],
+                                s_r[cb][3 * q], s_r[cb][3 * q + 1], s_r[cb][3 * q + 2], S, bits);
+            }
+            continue;
+        }
+        if (clipped) bits |= LW_ST_CLIP;
+        for (long long t = (long long)blockIdx.z * kFp64Threads + threadIdx.x; t < T;
+             t += (long long)gridDim.z * kFp64Threads) {
+            int sl = 0;   // the last pixel whose offset is <= t
 #pragma unroll
-                    for (int step = 16; step > 0; step >>= 1)
-                        if (s_kp[wslot + pos + step] <= t) pos += step;
-                    const int sl = wslot + pos;
-                    job(sl, s_ja[sl] + (t - s_kp[sl]));
+            for (int step = kFp64Threads / 2; step > 0; step >>= 1)
+                if (s_off[sl + step] <= t) sl += step;
+            const double n0 = s_n[sl][0], n1 = s_n[sl][1], n2 = s_n[sl][2];
+            const int j = s_ja[sl] + (int)(t - s_off[sl]);
+            const double J = (double)j;
+            // u - j of a sample, to FP32 rounding of its size and of the transverse terms':
+            // tau = t - z/c0 in FP64, n . r - z in FP32
+            const float wx = s_w[sl][0], wy = s_w[sl][1], wz = s_w[sl][2];
+            const double off = -fma(p.t_min, p.inv_dtu, J);
+            auto ahead = [&](int g) -> float {
+                const double* x = rk + 3 * (int64_t)g;
+                const double d = fma(fma(-x[2], kInvC0, tk[g]), p.inv_dtu, off);
+                return fmaf(wx, to_float(x[0]),
+                            fmaf(wy, to_float(x[1]), fmaf(wz, to_float(x[2]), to_float(d))));
+            };
+            int ia = 0, ib = last;   // u(ia) < j <= u(ib)
+            float xa = to_float(s_u[sl][0] - J), xb = to_float(s_u[sl][1] - J);
+            for (int probes = 0; ib - ia > 1; ++probes) {
+                int g = ia + ((ib - ia) >> 1);
+                if (probes < kFalsiProbes) {
+                    const float gf = ceilf(__fdividef(xa, xa - xb) * (float)(ib - ia));
+                    g = ia + (int)fminf(fmaxf(gf, 1.0f), (float)(ib - ia - 1));
+                }
+                const float x = ahead(g);
+                if (x >= 0.0f) {
+                    ib = g;
+                    xb = x;
+                } else {
+                    ia = g;
+                    xa = x;
                 }
             }
-            for (int t = 0; t < big; ++t) job(threadIdx.x, ja + t);   // runs beyond the warp count
-            __syncwarp();
+            auto time = [&](int g) {
+                const double* x = rk + 3 * (int64_t)g;
+                return advanced_time_fp64(n0, n1, n2, x[0], x[1], x[2], tk[g]);
+            };
+            // the first sample that reaches j by the scan's coordinate: the search can be off by
+            // the FP32 rounding; u(0) < j <= u(last) bound both walks
+            double ta = time(ib), tb = time(ia);
+            while (ib < last && coord(ta) < J) {
+                tb = ta;
+                ia = ib++;
+                ta = time(ib);
+            }
+            while (ia > 0 && coord(tb) >= J) {
+                ta = tb;
+                ib = ia--;
+                tb = time(ia);
+            }
+            double Fb[3], Fa[3];
+            field_fp64(n0, n1, n2, p.R, p.flags, bk + 3 * (int64_t)ia, ak + 3 * (int64_t)ia, Fb);
+            field_fp64(n0, n1, n2, p.R, p.flags, bk + 3 * (int64_t)ib, ak + 3 * (int64_t)ib, Fa);
+            const double den = __dsub_rn(ta, tb);
+            deposit_fp64(p, static_cast<double*>(p.record) + (pix0 + sl) * 3 * p.n_bins + j, J, ta,
+                         tb, den, __drcp_rn(den), Fa, Fb);
         }
     }
     cp_async_wait_all();
@@ -1430,8 +1438,14 @@ extern "C" int lw_deposit_time_domain(const lw_traj* traj, const lw_detector* de
     if (precision == LW_FP64) {
         const int64_t tiles = (det->n_pix + kFp64Threads - 1) / kFp64Threads;
         a.e_chunk = (int)std::max<int64_t>(1, (traj->n_e + 65534) / 65535);
-        dim3 g((unsigned)tiles, (unsigned)((traj->n_e + a.e_chunk - 1) / a.e_chunk));
-        deposit_fp64_jobs_kernel<<<g, kFp64Threads, 0, st>>>(a);
+        const int64_t rows = (traj->n_e + a.e_chunk - 1) / a.e_chunk;
+        // an electron's steps (or grid points) are divided over grid z until there are about
+        // 24 CTAs per SM: four are resident, and a last wave of 64 electrons x 400 pixels at
+        // two waves' worth of CTAs left most SMs idle
+        const int64_t nblk = (traj->n_s + kF64Block) / kF64Block;
+        const int64_t parts = std::min<int64_t>(nblk, (kSms * 24 + tiles * rows - 1) / (tiles * rows));
+        dim3 g((unsigned)tiles, (unsigned)rows, (unsigned)std::min<int64_t>(parts, 65535));
+        deposit_fp64_kernel<<<g, kFp64Threads, 0, st>>>(a);
         return launch_status();
     }
     constexpr int PIX = kMixPix;
