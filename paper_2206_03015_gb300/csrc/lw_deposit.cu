@@ -298,15 +298,13 @@ __device__ __forceinline__ DF split_double(double x) {
     return r;
 }
 
-// Compensated atomic accumulation into a (sum, compensation) pair: the
-// rounding error of the atomic add is recovered exactly from the returned old
-// value (two-sum) and added to the compensation word.
-__device__ __forceinline__ void kahan_atomic_add(float2* p, float v) {
-    const float old = atomicAdd(&p->x, v);
+// Compensated accumulation into a (sum, compensation) pair: the rounding error of the atomic
+// addition of v is recovered exactly from the returned old value (two-sum) and added to the
+// compensation word.
+__device__ __forceinline__ float two_sum_error(float old, float v) {
     const float s = __fadd_rn(old, v);
     const float bb = __fsub_rn(s, old);
-    const float err = __fadd_rn(__fsub_rn(old, __fsub_rn(s, bb)), __fsub_rn(v, bb));
-    if (err != 0.0f) atomicAdd(&p->y, err);
+    return __fadd_rn(__fsub_rn(old, __fsub_rn(s, bb)), __fsub_rn(v, bb));
 }
 
 struct PixelConst {
@@ -402,9 +400,7 @@ enum { kAccF64 = 0, kAccKahan = 1, kAccF32 = 2, kAccF32X4 = 3 };
 
 template <int ACC>
 __device__ __forceinline__ void accumulate(void* rec, int64_t idx, float v) {
-    if (ACC == kAccKahan) {
-        kahan_atomic_add(static_cast<float2*>(rec) + idx, v);
-    } else if (ACC == kAccF32) {
+    if (ACC == kAccF32) {
         atomicAdd(static_cast<float*>(rec) + idx, v);
     } else {
         atomicAdd(static_cast<double*>(rec) + idx, (double)v);
@@ -421,6 +417,19 @@ __device__ __forceinline__ void deposit3_row(unsigned char* row, int j, int64_t 
         asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v0),
                      "f"(v1), "f"(v2), "f"(0.0f)
                      : "memory");
+    } else if (ACC == kAccKahan) {
+        // the three returning additions first, so that their round trips to the L2 overlap, and
+        // the errors with one predicate each (999 electrons x 3,001 steps x 1,517 pixels, 6 additions
+        // a bin: 11.5 -> 8.1 ms)
+        float2* p = reinterpret_cast<float2*>(row) + j;
+        const float o0 = atomicAdd(&p->x, v0);
+        const float o1 = atomicAdd(&p[n_bins].x, v1);
+        const float o2 = atomicAdd(&p[2 * n_bins].x, v2);
+        const float e0 = two_sum_error(o0, v0), e1 = two_sum_error(o1, v1),
+                    e2 = two_sum_error(o2, v2);
+        if (e0 != 0.0f) atomicAdd(&p->y, e0);
+        if (e1 != 0.0f) atomicAdd(&p[n_bins].y, e1);
+        if (e2 != 0.0f) atomicAdd(&p[2 * n_bins].y, e2);
     } else {
         accumulate<ACC>(row, j, v0);
         accumulate<ACC>(row, j + n_bins, v1);
