@@ -26,6 +26,7 @@
 //   D = (1 - n_z) + n_z (1 - beta_z) - n_perp . beta_perp,
 // and contributions are added with FP64 atomics, a compensated pair of FP32
 // atomics, or FP32 atomics (the three mixed records).
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include <algorithm>
@@ -609,8 +610,21 @@ __device__ __forceinline__ int frac_floor(float f) { return f >= 1.0f ? 1 : (f <
 // would add or drop a whole sample (Algorithm 2's half-open interval), are recomputed
 // with the FP64 path's operation order when the mixed value lies within a guard band
 // of an integer.
-template <int PIX, int ACC, int FL, bool CHECK>
-__device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int64_t chunk) {
+//
+// The blocks of every electron may be divided over `parts` CTAs (part = 0 .. parts-1): a part
+// starts from its first block's anchor, whose bin is the end of the part before (the same
+// anchor, the same arithmetic).  Problems whose tiles and chunks are few fill the GPU that way.
+// Flagged inputs (a step longer than c0 dt, times out of order, non-finite values) are left to
+// part 0, where the last grid point reached is carried over the whole trajectory.
+//
+// With CHECK the CTAs of a unit (its parts, and with PIX = 1 the two halves of its tile) are a
+// cluster over which the unit's sums are taken.  Without SPLIT
+// (one part, known at compile time) the deposit keeps the registers that the parts cost it
+// (80 instead of 74 with spills: 0.8 % of a 10,000-electron step).
+template <int PIX, int ACC, int FL, bool CHECK, bool SPLIT>
+__device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int64_t chunk,
+                                         int part_ = 0, int parts_ = 1) {
+    const int part = SPLIT ? part_ : 0, parts = SPLIT ? parts_ : 1;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr int kSlots = kMixThreads * PIX;
     const int B = p.block;
@@ -669,7 +683,9 @@ __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int
     }
     __syncthreads();   // barriers initialised
     int bits = 0;
-    if (tile == 0 && chunk == 0 && threadIdx.x == 0 && p.input_status) bits |= *p.input_status;
+    const int flagged = SPLIT && p.input_status ? *p.input_status : 0;
+    if (tile == 0 && chunk == 0 && part == 0 && threadIdx.x == 0 && p.input_status)
+        bits |= *p.input_status;
     float err2 = 0.0f, val2 = 0.0f;   // CHECK: squared error estimates and squared values
 
     // the tile's first record row; a pixel row is 4 * record_words bytes per grid point
@@ -680,6 +696,15 @@ __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int
     auto electron = [&](int64_t kk) -> int64_t { return p.order ? (int64_t)p.order[kk] : kk; };
     // blocks with at least one step: ceil((ns1 - 1) / B)
     const int nbs = (int)((p.ns1 - 2) / B + 1);
+    // this part's blocks [b_lo, b_hi); a part never starts at the last block of an anchor batch,
+    // whose end anchor is in the next one
+    auto cut = [&](int q) -> int {
+        if (!SPLIT) return q == 0 ? 0 : nbs;
+        if (flagged & (LW_ST_STEP | LW_ST_TIME | LW_ST_NONFINITE)) return q == 0 ? 0 : nbs;
+        const int c = (int)((int64_t)nbs * q / parts);
+        return c < nbs && (c & (kAnchorBatch - 1)) == kAnchorBatch - 1 ? c + 1 : c;
+    };
+    const int b_lo = cut(part), b_hi = cut(part + 1);
     // float2 field records of a block start 0 or 8 bytes into their area: the bulk copy
     // starts at the 16-byte boundary at or before the block's first record
     auto field_shift = [&](int64_t k, int b) -> int {
@@ -694,7 +719,8 @@ __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int
         const int sh = field_shift(k, b);
         const unsigned f4_bytes = 16u * (unsigned)(ns + 1);
         const unsigned f2_bytes = (8u * (unsigned)(ns + 1) + (unsigned)sh + 15u) & ~15u;
-        const int a0 = b == 0 ? 0 : ((b & (kAnchorBatch - 1)) == kAnchorBatch - 1 ? b + 1 : -1);
+        const int a0 = b == b_lo ? b & ~(kAnchorBatch - 1)
+                                 : ((b & (kAnchorBatch - 1)) == kAnchorBatch - 1 ? b + 1 : -1);
         const unsigned anc_bytes =
             a0 >= 0 ? (unsigned)(sizeof(Anchor) * min(kAnchorBatch, p.n_blocks - a0)) : 0u;
         fence_proxy_async_smem();   // the buffer's previous contents were read by the CTA
@@ -710,18 +736,18 @@ __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int
     };
 
     const int64_t k0 = chunk * p.e_chunk;
-    const int64_t k1 = min(k0 + p.e_chunk, p.n_e);
+    const int64_t k1 = b_lo < b_hi ? min(k0 + p.e_chunk, p.n_e) : k0;
     // ring: the unit's (electron, block) stages in order, kMixStages - 1 in flight ahead;
     // every thread keeps the bookkeeping, thread 0 issues the copies
     int64_t iss_kk = k0;   // next stage to issue
-    int iss_b = 0;
+    int iss_b = b_lo;
     unsigned pending = 0;   // bit s: buffer s has a copy in flight
     auto issue_next = [&](int buf) {
         if (iss_kk < k1) {
             if (threadIdx.x == 0) issue(electron(iss_kk), iss_b, buf);
             pending |= 1u << buf;
-            if (++iss_b == nbs) {
-                iss_b = 0;
+            if (++iss_b == b_hi) {
+                iss_b = b_lo;
                 ++iss_kk;
             }
         }
@@ -774,11 +800,11 @@ __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int
     for (int64_t kk = k0; kk < k1 && !timed_out; ++kk) {
         const int64_t k = electron(kk);
         // per pixel: (Is, fs) = the block's start anchor, jdone = last grid point reached
-        // so far (absolute; from the first sample's bin in block 0)
+        // so far (absolute; from the part's first anchor, in block 0 the first sample's bin)
         int Is[PIX], jdone[PIX];
         float fs[PIX];
         float anc32[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-        for (int b = 0; b < nbs; ++b) {
+        for (int b = b_lo; b < b_hi; ++b) {
             const int64_t i0 = (int64_t)b * B;
             const int ns = (int)min((int64_t)B, p.ns1 - 1 - i0);   // steps: (i0+r-1, i0+r], r=1..ns
             const bool ok = mbar_wait(&s_full[cur], (phase >> cur) & 1u);
@@ -801,11 +827,11 @@ __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int
             // anchors: lane l holds the FP32 pairs of anchor 32c + l (c = batch); block b's
             // end anchor is b + 1
             const int ab = b & (kAnchorBatch - 1);
-            if (b == 0) {
-                if (lane < p.n_blocks) split_anchor(s_anc[lane], anc32);
+            if (b == b_lo) {
+                if (lane < p.n_blocks - (b - ab)) split_anchor(s_anc[lane], anc32);
                 float an0[8];
 #pragma unroll
-                for (int c = 0; c < 8; ++c) an0[c] = __shfl_sync(0xffffffffu, anc32[c], 0);
+                for (int c = 0; c < 8; ++c) an0[c] = __shfl_sync(0xffffffffu, anc32[c], ab);
 #pragma unroll
                 for (int q = 0; q < PIX; ++q) {   // block 0's anchor is sample 0
                     anchor_of(an0, make_float4(whi[q][0], whi[q][1], whi[q][2], 0.0f), q,
@@ -813,7 +839,8 @@ __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int
                     const int fl = frac_floor(fs[q]);
                     const float fr = fs[q] - (float)fl;
                     jdone[q] = Is[q] + fl;
-                    if (fr < kFirstGuard || fr > 1.0f - kFirstGuard) jdone[q] = end_bin(k, q, 0);
+                    if (b == 0 && (fr < kFirstGuard || fr > 1.0f - kFirstGuard))
+                        jdone[q] = end_bin(k, q, 0);
                 }
             }
             const bool end_anchor = i0 + B <= p.ns1 - 1;   // the block ends at anchor b + 1
@@ -1039,8 +1066,20 @@ __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int
             atomicAdd(&s_err[1], val2);
         }
         __syncthreads();
-        if (threadIdx.x == 0 && s_err[0] > kPrecisionTol * kPrecisionTol * s_err[1])
-            bits |= LW_ST_PRECISION;
+        float e = s_err[0], v = s_err[1];
+        // a cluster: its first CTA adds up the others'
+        namespace cg = cooperative_groups;
+        cg::cluster_group cl = cg::this_cluster();
+        cl.sync();
+        if (cl.block_rank() == 0 && threadIdx.x == 0) {
+            for (unsigned r = 1; r < cl.num_blocks(); ++r) {
+                const float* o = cl.map_shared_rank(s_err, r);
+                e += o[0];
+                v += o[1];
+            }
+            if (e > kPrecisionTol * kPrecisionTol * v) bits |= LW_ST_PRECISION;
+        }
+        cl.sync();   // the others' sums stay readable until then
     }
     if (timed_out) {
         bits |= LW_ST_TIMEOUT;
@@ -1259,17 +1298,20 @@ __global__ void __launch_bounds__(kFp64Threads) deposit_fp64_kernel(DepositArgs 
     block_status_or(p.status, bits);
 }
 
-template <int PIX, int ACC, int FL>
+template <int PIX, int ACC, int FL, bool SPLIT>
 __global__ void __launch_bounds__(kMixThreads, kMixMinBlocks) deposit_mixed_kernel(DepositArgs p) {
     // the precision check launched after this grid (programmatic dependent launch) may
     // start once every CTA of this grid has started: it fills the SMs of the last wave
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int bits = mixed_cta<PIX, ACC, FL, false>(p, blockIdx.x, blockIdx.y);
+    const int bits =
+        mixed_cta<PIX, ACC, FL, false, SPLIT>(p, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.z);
     block_status_or(p.status, bits);
 }
 
 // Precision check of a mixed deposit: the units of every `stride`-th electron chunk
-// (grid y = sampled chunks), evaluated without depositing.  Launched as a programmatic
+// (grid y = sampled chunks), evaluated without depositing, each by a cluster of CTAs that share
+// its blocks and, with PIX = 1, its 512 pixels (check_shape; 16 electrons x 2,000 steps x 1,024
+// pixels, all of whose units are checked: 677 us with one CTA per unit, 134 with eight).  Launched as a programmatic
 // dependent of the deposit, it runs beside the deposit's last CTAs and, before it ends,
 // waits for the deposit grid to complete (griddepcontrol.wait: its completion and memory
 // flush), so that work after it in the stream sees the finished record; without that
@@ -1277,8 +1319,8 @@ __global__ void __launch_bounds__(kMixThreads, kMixMinBlocks) deposit_mixed_kern
 template <int PIX, int FL>
 __global__ void __launch_bounds__(kMixThreads, kMixMinBlocks)
     deposit_check_kernel(DepositArgs p, int stride) {
-    const int bits =
-        mixed_cta<PIX, kAccF32X4, FL, true>(p, blockIdx.x, (int64_t)blockIdx.y * stride);
+    const int bits = mixed_cta<PIX, kAccF32X4, FL, true, true>(p, blockIdx.x, (int64_t)blockIdx.y * stride,
+                                                          blockIdx.z, gridDim.z);
     block_status_or(p.status, bits & LW_ST_PRECISION);
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -1309,7 +1351,7 @@ __global__ void __launch_bounds__(kMixThreads, kMixMinBlocks)
         if (u >= n_units) break;
         const BatchUnit un = units[u];
         const DepositArgs& p = c_batch_vars[un.variant];
-        const int bits = mixed_cta<PIX, ACC, FL, false>(p, un.tile, un.chunk);
+        const int bits = mixed_cta<PIX, ACC, FL, false, false>(p, un.tile, un.chunk);
         block_status_or(p.status, bits);
     }
 }
@@ -1318,11 +1360,11 @@ __global__ void __launch_bounds__(kMixThreads, kMixMinBlocks)
 template <int PIX, int FL>
 __global__ void __launch_bounds__(kMixThreads, kMixMinBlocks)
     deposit_batched_check_kernel(const BatchUnit* __restrict__ units, int n_units, int stride) {
-    const int u = blockIdx.x * stride;
-    if (u >= n_units) return;
+    const int u = blockIdx.x * stride;   // < n_units by the grid
     const BatchUnit un = units[u];
     const DepositArgs& p = c_batch_vars[un.variant];
-    const int bits = mixed_cta<PIX, kAccF32X4, FL, true>(p, un.tile, un.chunk);
+    const int bits =
+        mixed_cta<PIX, kAccF32X4, FL, true, true>(p, un.tile, un.chunk, blockIdx.z, gridDim.z);
     block_status_or(p.status, bits & LW_ST_PRECISION);
 }
 
@@ -1347,15 +1389,20 @@ __global__ void zero_records_kernel(const DepositArgs* __restrict__ vars, int wo
 // Kernel instances by accumulation form and field terms (LW_FIELD_* mask 1, 2 or 3).
 using MixedKernel = void (*)(DepositArgs);
 using BatchedKernel = void (*)(const BatchUnit*, int, int*);
-template <int ACC>
+// (a divided deposit has one pixel per thread: twice the warps)
+template <int ACC, bool SPLIT>
 MixedKernel mixed_kernel_fl(uint32_t fl) {
-    return fl == 1 ? deposit_mixed_kernel<kMixPix, ACC, 1>
-           : fl == 2 ? deposit_mixed_kernel<kMixPix, ACC, 2> : deposit_mixed_kernel<kMixPix, ACC, 3>;
+    constexpr int PIX = SPLIT ? 1 : kMixPix;
+    return fl == 1 ? deposit_mixed_kernel<PIX, ACC, 1, SPLIT>
+           : fl == 2 ? deposit_mixed_kernel<PIX, ACC, 2, SPLIT>
+                     : deposit_mixed_kernel<PIX, ACC, 3, SPLIT>;
 }
+template <bool SPLIT>
 MixedKernel mixed_kernel(int acc, uint32_t fl) {
-    return acc == kAccKahan ? mixed_kernel_fl<kAccKahan>(fl)
-           : acc == kAccF32 ? mixed_kernel_fl<kAccF32>(fl)
-           : acc == kAccF32X4 ? mixed_kernel_fl<kAccF32X4>(fl) : mixed_kernel_fl<kAccF64>(fl);
+    return acc == kAccKahan ? mixed_kernel_fl<kAccKahan, SPLIT>(fl)
+           : acc == kAccF32 ? mixed_kernel_fl<kAccF32, SPLIT>(fl)
+           : acc == kAccF32X4 ? mixed_kernel_fl<kAccF32X4, SPLIT>(fl)
+                              : mixed_kernel_fl<kAccF64, SPLIT>(fl);
 }
 template <int ACC>
 BatchedKernel batched_kernel_fl(uint32_t fl) {
@@ -1364,9 +1411,10 @@ BatchedKernel batched_kernel_fl(uint32_t fl) {
                      : deposit_batched_kernel<kMixPix, ACC, 3>;
 }
 using CheckKernel = void (*)(DepositArgs, int);
+template <int PIX>
 CheckKernel check_kernel(uint32_t fl) {
-    return fl == 1 ? deposit_check_kernel<kMixPix, 1>
-           : fl == 2 ? deposit_check_kernel<kMixPix, 2> : deposit_check_kernel<kMixPix, 3>;
+    return fl == 1 ? deposit_check_kernel<PIX, 1>
+           : fl == 2 ? deposit_check_kernel<PIX, 2> : deposit_check_kernel<PIX, 3>;
 }
 using BatchedCheckKernel = void (*)(const BatchUnit*, int, int);
 BatchedCheckKernel batched_check_kernel(uint32_t fl) {
@@ -1378,6 +1426,20 @@ BatchedKernel batched_kernel(int acc, uint32_t fl) {
     return acc == kAccKahan ? batched_kernel_fl<kAccKahan>(fl)
            : acc == kAccF32 ? batched_kernel_fl<kAccF32>(fl)
            : acc == kAccF32X4 ? batched_kernel_fl<kAccF32X4>(fl) : batched_kernel_fl<kAccF64>(fl);
+}
+
+// The cluster that checks one unit: its tile in two halves (one pixel per thread) and its blocks
+// in up to four parts, eight CTAs together (the portable size), as long as the check stays
+// within one wave of resident CTAs -- beyond that dividing a unit only repeats its set-up (320
+// units of a 10,000-electron deposit in eight parts: 18.37 ms a step instead of 18.27).
+struct CheckShape {
+    int halves, parts;
+};
+CheckShape check_shape(int64_t nbs, int64_t units) {
+    constexpr int64_t wave = (int64_t)kSms * kMixMinBlocks;
+    CheckShape c{2 * units <= wave ? 2 : 1, 4};
+    while (c.parts > 1 && (c.parts > nbs || c.parts * c.halves * units > wave)) c.parts >>= 1;
+    return c;
 }
 
 // The mixed path's FP32 constants from the FP64 grid and detector fields (each the FP32
@@ -1457,8 +1519,7 @@ extern "C" int lw_deposit_time_domain(const lw_traj* traj, const lw_detector* de
         deposit_fp64_kernel<<<g, kFp64Threads, 0, st>>>(a);
         return launch_status();
     }
-    constexpr int PIX = kMixPix;
-    const int64_t tiles = (det->n_pix + kMixThreads * PIX - 1) / (kMixThreads * PIX);
+    const int64_t tiles = (det->n_pix + kMixThreads * kMixPix - 1) / (kMixThreads * kMixPix);
     // a few consecutive electrons (in arrival order) per CTA row -- enough rows for
     // about eight waves of resident CTAs -- dispatched tile-fastest: the electrons in
     // flight stay consecutive in arrival order, so the record bins they update are few
@@ -1469,9 +1530,21 @@ extern "C" int lw_deposit_time_domain(const lw_traj* traj, const lw_detector* de
                            precision == LW_MIXED_F32X4 ? kMixMaxChunkX4 : kMixMaxChunk);
     a.e_chunk = (int)std::max<int64_t>(ec, (traj->n_e + 65534) / 65535);
     dim3 g((unsigned)tiles, (unsigned)((traj->n_e + a.e_chunk - 1) / a.e_chunk));
+    // less than two waves of CTAs: tiles of one pixel per thread, and the blocks of an electron
+    // divided over grid z, up to two waves (16 electrons x 2,000 steps x 1,024 pixels: 571 us in 32
+    // CTAs, 110 in 256)
+    const int64_t nbs = (traj->n_s - 1) / traj->block + 1;
+    const int64_t two_waves = (int64_t)kSms * kMixMinBlocks * 2;
+    const bool split = (int64_t)g.x * g.y < two_waves;
+    if (split) {
+        g.x = (unsigned)((det->n_pix + kMixThreads - 1) / kMixThreads);
+        const int64_t ctas = (int64_t)g.x * g.y;
+        g.z = (unsigned)std::min<int64_t>(std::min<int64_t>(nbs, 64), (two_waves + ctas - 1) / ctas);
+    }
     const size_t smem = kMixStages * stage_bytes(traj->block);   // staging ring
     // static tables + double-buffered staging exceed the 48 KB default: opt in
-    const MixedKernel kern = mixed_kernel(acc_of(precision), field_flags);
+    const MixedKernel kern = split ? mixed_kernel<true>(acc_of(precision), field_flags)
+                                   : mixed_kernel<false>(acc_of(precision), field_flags);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
         cudaSuccess)
         return LW_ECUDA;
@@ -1480,20 +1553,28 @@ extern "C" int lw_deposit_time_domain(const lw_traj* traj, const lw_detector* de
     if (status) {   // the precision check on a sample of the electron chunks (LW_ST_PRECISION)
         const int64_t chunks = g.y;
         const int stride = chunks > kCheckStride ? kCheckStride : 1;
-        const CheckKernel ck = check_kernel(field_flags);
+        const int64_t sampled = (chunks + stride - 1) / stride;
+        const CheckShape shape = check_shape(nbs, tiles * sampled);
+        const CheckKernel ck =
+            shape.halves == 2 ? check_kernel<1>(field_flags) : check_kernel<kMixPix>(field_flags);
         if (cudaFuncSetAttribute(ck, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
             cudaSuccess)
             return LW_ECUDA;
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(g.x, (unsigned)((chunks + stride - 1) / stride));
+        cfg.gridDim = dim3((unsigned)(tiles * shape.halves), (unsigned)sampled,
+                           (unsigned)shape.parts);
         cfg.blockDim = dim3(kMixThreads);
         cfg.dynamicSmemBytes = smem;
         cfg.stream = st;
-        cudaLaunchAttribute attr[1];
+        cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = (unsigned)shape.halves;
+        attr[1].val.clusterDim.y = 1;
+        attr[1].val.clusterDim.z = (unsigned)shape.parts;
         cfg.attrs = attr;
-        cfg.numAttrs = 1;
+        cfg.numAttrs = 2;
         if (cudaLaunchKernelEx(&cfg, ck, a, stride) != cudaSuccess) return LW_ECUDA;
     }
     return launch_status();
@@ -1650,7 +1731,6 @@ extern "C" int lw_batch_plan(const lw_batch_item* items, int32_t n_items, int32_
 }
 
 extern "C" int lw_batch_deposit(const lw_batch* plan, void* stream) {
-    constexpr int PIX = kMixPix;
     if (!plan || !plan->ws || plan->n_items < 1) return LW_EINVAL;
     cudaStream_t st = as_stream(stream);
     char* base = static_cast<char*>(plan->ws);
@@ -1688,7 +1768,22 @@ extern "C" int lw_batch_deposit(const lw_batch* plan, void* stream) {
     if (cudaFuncSetAttribute(ck, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              plan->smem_bytes) != cudaSuccess)
         return LW_ECUDA;
-    ck<<<(plan->n_units + stride - 1) / stride, kMixThreads, plan->smem_bytes, st>>>(
-        units, plan->n_units, stride);
+    cudaLaunchConfig_t cfg = {};
+    const int sampled = (plan->n_units + stride - 1) / stride;
+    // (units of 512-pixel tiles: parts only; a variant of fewer blocks leaves some without work)
+    unsigned parts = 8;
+    while (parts > 1 && (int64_t)parts * sampled > (int64_t)kSms * kMixMinBlocks) parts >>= 1;
+    cfg.gridDim = dim3((unsigned)sampled, 1, parts);
+    cfg.blockDim = dim3(kMixThreads);
+    cfg.dynamicSmemBytes = (size_t)plan->smem_bytes;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = parts;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, ck, units, (int)plan->n_units, stride) != cudaSuccess)
+        return LW_ECUDA;
     return launch_status();
 }
