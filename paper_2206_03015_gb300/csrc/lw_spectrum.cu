@@ -201,17 +201,19 @@ __global__ void pass_twiddle_kernel(typename V2<T>::type* tw, int logN) {
     }
 }
 
-// R-point transform (sign +) in registers; output k is left in x[rev(k)].
+// R-point transform (sign +) in registers of inputs in bit-reversed order: radix-2 stages with
+// constant roots, in the order of fft_pass.
 template <typename C, int R>
 __device__ __forceinline__ void fft_regs(C* x) {
 #pragma unroll
-    for (int half = R / 2; half >= 1; half >>= 1) {
+    for (int half = 1; half < R; half <<= 1) {
 #pragma unroll
         for (int m = 0; m < R; ++m) {
             if (m & half) continue;
-            const C u = x[m], v = x[m + half];
+            const C v = mul_root16(x[m + half], (m & (half - 1)) * (8 / half));
+            const C u = x[m];
             x[m] = cadd(u, v);
-            x[m + half] = mul_root16(csub(u, v), (m & (half - 1)) * (8 / half));
+            x[m + half] = csub(u, v);
         }
     }
 }
@@ -229,7 +231,7 @@ struct RegPlan {
 __device__ __forceinline__ int reg_slot(int j) { return j + (j >> 4); }
 
 // Passes from LOGNS on over v (in: element t + i N/16 of the pass's input is v[i]); the last
-// pass's output stays in v with element index tb + r N/R at v[b R + rev(r)].
+// pass's output is left in the buffer in natural order.
 template <typename C, int LOGN, int LOGNS>
 __device__ __forceinline__ void reg_passes(C* v, C* buf, const C* __restrict__ tw) {
     constexpr int N = 1 << LOGN, T = N / 16;
@@ -242,11 +244,12 @@ __device__ __forceinline__ void reg_passes(C* v, C* buf, const C* __restrict__ t
 #pragma unroll
     for (int b = 0; b < M; ++b) {
 #pragma unroll
-        for (int i = 0; i < R; ++i) {
-            x[b * R + i] = v[b + i * M];
+        for (int m = 0; m < R; ++m) {
+            const int i = rev_bits(m, LOGR);
+            x[b * R + m] = v[b + i * M];
             if (LOGNS > 0 && i > 0) {
                 const int q = (t + b * T) & (Ns - 1);
-                x[b * R + i] = cmul(x[b * R + i], tw[(i - 1) * Ns + q]);
+                x[b * R + m] = cmul(x[b * R + m], tw[(i - 1) * Ns + q]);
             }
         }
         fft_regs<C, R>(x + b * R);
@@ -258,7 +261,7 @@ __device__ __forceinline__ void reg_passes(C* v, C* buf, const C* __restrict__ t
             const int tb = t + b * T;
             const int d = ((tb >> LOGNS) << (LOGNS + LOGR)) + (tb & (Ns - 1));
 #pragma unroll
-            for (int r = 0; r < R; ++r) buf[reg_slot(d + r * Ns)] = x[b * R + rev_bits(r, LOGR)];
+            for (int r = 0; r < R; ++r) buf[reg_slot(d + r * Ns)] = x[b * R + r];
         }
         __syncthreads();
 #pragma unroll
@@ -270,7 +273,7 @@ __device__ __forceinline__ void reg_passes(C* v, C* buf, const C* __restrict__ t
         for (int b = 0; b < M; ++b)
 #pragma unroll
             for (int r = 0; r < R; ++r)
-                buf[reg_slot(t + b * T + r * (N / R))] = x[b * R + rev_bits(r, LOGR)];
+                buf[reg_slot(t + b * T + r * (N / R))] = x[b * R + r];
         __syncthreads();
     }
 }
@@ -584,7 +587,11 @@ int run_spectrum(const void* record, int kind, int64_t n_pix, const lw_grid* g, 
     // records, one CTA per pair against four-step: 2,048 pixels x 16,384 bins 296 and 477 us,
     // 400 pixels 81 and 107, 200 pixels 42 and 59, 100 pixels 40 and 37; 8,192 bins and 200
     // pixels 37 and 37, 400 pixels 39 and 57.  FP64 at 8,192 bins: 400 pixels 742 and 579.
-    const bool regs = N >= 1024 && (N <= 4096 || (sizeof(T) == 4 && N <= 16384 &&
+    // Four-step too where X' is kept for a gradient: FP32 transforms that round in another order
+    // moved a mixed gradient's residuals (dL/da0 by 1.8e-7, twelve times its run-to-run noise),
+    // and a transform is 0.1 % of a gradient step.  (Up to 4,096 bins the registers' passes
+    // round as those in shared memory do.)
+    const bool regs = N >= 1024 && (N <= 4096 || (sizeof(T) == 4 && N <= 16384 && !X_save &&
                                                   (n_pix + 1) / 2 >= kSms / 2));
     const bool direct = N <= 4096;
     const int64_t n_pairs = (n_pix + 1) / 2;
