@@ -372,6 +372,12 @@ __global__ void __launch_bounds__(kAdjThreads) adj_deposit_kernel(AdjArgs p) {
 
 // ------------------------------------------------------------ mixed-precision adjoint
 //
+// (2,048 electrons x 4,096 steps x 1,024 pixels x 16,384 bins: 269 ms with 64-bit grid indices,
+// whose conversions held the FP64 pipe at 71 %, a second field evaluation in the chain rule and
+// 45 shuffles per sample; 32-bit indices, one evaluation and warp_sum9 take 197 ms.  What
+// remains is latency: 54 % of the issue slots at 5 warps per scheduler, long scoreboard on the
+// record gradient's rows.)
+//
 // The same transpose in mixed precision: the bin coordinate of each tile's first sample in
 // FP64 and, within the tile of 64 samples, each sample's as an integer plus an FP32
 // fraction advanced by the step's FP32 increment (from FP64-differenced samples), so the
@@ -420,68 +426,57 @@ struct NF {   // a pixel direction in FP32 with 1 - n_z kept exactly
     float x, y, z, omz;
 };
 
-// acceleration field (n - beta) (n . bdot) - D bdot) / D^3 in FP32; zero when |beta| >= 1
-// (b.w == 0) or D <= 0
-__device__ __forceinline__ void field_acc_f32(const NF& n, float4 b, float4 a, float F[3]) {
-    const float D = fmaf(-n.y, b.y, fmaf(-n.x, b.x, fmaf(n.z, b.z, n.omz)));
-    const float mx = n.x - b.x, my = n.y - b.y, mz = b.z - n.omz;
-    const float nbd = fmaf(n.z, a.z, fmaf(n.y, a.y, n.x * a.x));
-    const float iD = __fdividef(1.0f, D);
-    const float iD3 = (b.w != 0.0f && D > 0.0f) ? iD * iD * iD : 0.0f;
-    F[0] = fmaf(mx, nbd, -D * a.x) * iD3;
-    F[1] = fmaf(my, nbd, -D * a.y) * iD3;
-    F[2] = fmaf(mz, nbd, -D * a.z) * iD3;
+// One sample seen from one pixel: acceleration field ((n - beta) (n . bdot) - D bdot) / D^3 in FP32
+// and what its chain rule shares with it; all zero when |beta| >= 1 (b.w == 0) or D <= 0
+struct SampleF {
+    float mx, my, mz, nbd, D, iD, iD3;
+    float F[3];
+};
+__device__ __forceinline__ void sample_field_f32(const NF& n, float4 b, float4 a, SampleF& f) {
+    f.D = fmaf(-n.y, b.y, fmaf(-n.x, b.x, fmaf(n.z, b.z, n.omz)));
+    f.mx = n.x - b.x;
+    f.my = n.y - b.y;
+    f.mz = b.z - n.omz;
+    f.nbd = fmaf(n.z, a.z, fmaf(n.y, a.y, n.x * a.x));
+    const bool ok = b.w != 0.0f && f.D > 0.0f;
+    f.iD = ok ? __fdividef(1.0f, f.D) : 0.0f;
+    f.iD3 = f.iD * f.iD * f.iD;
+    f.F[0] = fmaf(f.mx, f.nbd, -f.D * a.x) * f.iD3;
+    f.F[1] = fmaf(f.my, f.nbd, -f.D * a.y) * f.iD3;
+    f.F[2] = fmaf(f.mz, f.nbd, -f.D * a.z) * f.iD3;
 }
 
 // (dL/dF, dL/du_a) of one sample -> (dL/du_a n, dL/dbeta, dL/dbdot) in FP32, on the scale
 // of the record gradient; dL/dr = -(dL/du_a) n / (c0 dt_u) is completed by the caller
-__device__ __forceinline__ void sample_chain_f32(const NF& n, float4 b, float4 a,
+__device__ __forceinline__ void sample_chain_f32(const NF& n, const SampleF& f, float4 a,
                                                  const float G[3], float gu, float o[9]) {
     o[0] = gu * n.x;
     o[1] = gu * n.y;
     o[2] = gu * n.z;
-    const float D = fmaf(-n.y, b.y, fmaf(-n.x, b.x, fmaf(n.z, b.z, n.omz)));
-    if (b.w == 0.0f || !(D > 0.0f)) {
-        for (int c = 3; c < 9; ++c) o[c] = 0.0f;
-        return;
-    }
-    const float iD = __fdividef(1.0f, D), iD3 = iD * iD * iD;
-    const float mx = n.x - b.x, my = n.y - b.y, mz = b.z - n.omz;
-    const float nbd = fmaf(n.z, a.z, fmaf(n.y, a.y, n.x * a.x));
     const float bG = fmaf(a.z, G[2], fmaf(a.y, G[1], a.x * G[0]));
-    const float mG = fmaf(mz, G[2], fmaf(my, G[1], mx * G[0]));
-    const float Fx = fmaf(mx, nbd, -D * a.x) * iD3, Fy = fmaf(my, nbd, -D * a.y) * iD3,
-                Fz = fmaf(mz, nbd, -D * a.z) * iD3;
-    const float FG3 = 3.0f * fmaf(Fz, G[2], fmaf(Fy, G[1], Fx * G[0])) * iD;
-    o[3] = fmaf(fmaf(-nbd, G[0], n.x * bG), iD3, n.x * FG3);
-    o[4] = fmaf(fmaf(-nbd, G[1], n.y * bG), iD3, n.y * FG3);
-    o[5] = fmaf(fmaf(-nbd, G[2], n.z * bG), iD3, n.z * FG3);
-    o[6] = fmaf(n.x, mG, -D * G[0]) * iD3;
-    o[7] = fmaf(n.y, mG, -D * G[1]) * iD3;
-    o[8] = fmaf(n.z, mG, -D * G[2]) * iD3;
+    const float mG = fmaf(f.mz, G[2], fmaf(f.my, G[1], f.mx * G[0]));
+    const float FG3 = 3.0f * fmaf(f.F[2], G[2], fmaf(f.F[1], G[1], f.F[0] * G[0])) * f.iD;
+    o[3] = fmaf(fmaf(-f.nbd, G[0], n.x * bG), f.iD3, n.x * FG3);
+    o[4] = fmaf(fmaf(-f.nbd, G[1], n.y * bG), f.iD3, n.y * FG3);
+    o[5] = fmaf(fmaf(-f.nbd, G[2], n.z * bG), f.iD3, n.z * FG3);
+    o[6] = fmaf(n.x, mG, -f.D * G[0]) * f.iD3;
+    o[7] = fmaf(n.y, mG, -f.D * G[1]) * f.iD3;
+    o[8] = fmaf(n.z, mG, -f.D * G[2]) * f.iD3;
 }
 
-__device__ __forceinline__ void flush_sample_f32(const AdjArgs& p, bool act, const NF& n,
-                                                 int64_t k, int64_t i, float4 b, float4 a,
-                                                 const float G[3], float gu, bool nonzero,
-                                                 double r_scale, double u_scale) {
+__device__ __forceinline__ void flush_sample_f32(const AdjArgs& p, const NF& n, int64_t s,
+                                                 const SampleF& f, float4 a, const float G[3],
+                                                 float gu, bool nonzero) {
     if (!__any_sync(0xffffffffu, nonzero)) return;
     float o[9];
-    if (nonzero && act) {
-        sample_chain_f32(n, b, a, G, gu, o);
+    if (nonzero) {
+        sample_chain_f32(n, f, a, G, gu, o);
     } else {
         for (int c = 0; c < 9; ++c) o[c] = 0.0f;
     }
-    for (int c = 0; c < 9; ++c)
-        for (int s = 16; s > 0; s >>= 1) o[c] += __shfl_xor_sync(0xffffffffu, o[c], s);
-    if ((threadIdx.x & 31) == 0) {   // three 16-byte FP32 reductions (no FP64 in the loop)
-        float* f = p.f_grad + 12 * (k * p.ns1 + i);
-        asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(f), "f"(o[0]),
-                     "f"(o[1]), "f"(o[2]), "f"(o[3]) : "memory");
-        asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(f + 4), "f"(o[4]),
-                     "f"(o[5]), "f"(o[6]), "f"(o[7]) : "memory");
-        asm volatile("red.global.add.f32 [%0], %1;" ::"l"(f + 8), "f"(o[8]) : "memory");
-    }
+    int which;
+    const float v = warp_sum9(o, which);
+    if (which >= 0) atomicAdd(p.f_grad + 12 * s + which, v);   // one FP32 reduction of nine lanes
 }
 
 // the FP32 sums in FP64, unscaled, added to the caller's gradients
@@ -534,9 +529,6 @@ __global__ void __launch_bounds__(kAdjThreads) adj_deposit_mixed_kernel(AdjArgs 
     const double sw = kInvC0 * p.inv_dtu;
     const double wx = -nx * sw, wy = -ny * sw, wz = (1.0 - nz) * sw;
     const float s32 = (float)p.inv_dtu, wx32 = (float)wx, wy32 = (float)wy, wz32 = (float)wz;
-    const double r_scale = *p.rscale;
-    // dL/dr = -(dL/du_a) n / (c0 dt_u), on the record gradient's scale
-    const double u_scale = -r_scale * p.inv_dtu * kInvC0;
     const float* R = p.dLdrec_f + (active ? m * 3 * p.n_bins : 0);
     const bool vec = (p.n_bins & 3) == 0;
     // the FP64 adjoint's bin coordinate of a sample, and its split into floor + fraction
@@ -544,12 +536,15 @@ __global__ void __launch_bounds__(kAdjThreads) adj_deposit_mixed_kernel(AdjArgs 
         return __dmul_rn(__dsub_rn(advanced_time_fp64(nx, ny, nz, x, y, z, t), p.t_min),
                          p.inv_dtu);
     };
-    auto exact_coord = [&](double u, int64_t& Jo, float& fo) {
-        u = fmin(fmax(u, -1.0e15), 1.0e15);
+    // (32-bit integers: conversions from and to 64-bit ones run on the FP64 pipe, which ten of
+    // them per sample kept 71 % busy; coordinates are clamped to +-1e9, far beyond any grid)
+    auto exact_coord = [&](double u, int& Jo, float& fo) {
+        u = fmin(fmax(u, -1.0e9), 1.0e9);
         const double fl = floor(u);
-        Jo = (int64_t)fl;
+        Jo = (int)fl;
         fo = (float)(u - fl);
     };
+    const int nb1 = (int)p.n_bins - 1;
     const int64_t k0 = (int64_t)blockIdx.y * p.e_chunk;
     const int64_t k1 = min(k0 + p.e_chunk, p.n_e);
     for (int64_t k = k0; k < k1; ++k) {
@@ -557,17 +552,17 @@ __global__ void __launch_bounds__(kAdjThreads) adj_deposit_mixed_kernel(AdjArgs 
         const double* rk = p.r + 3 * k * p.ns1;
         const double* bk = p.beta + 3 * k * p.ns1;
         const double* ak = p.bdot + 3 * k * p.ns1;
-        float Fb[3] = {0.0f, 0.0f, 0.0f};
+        SampleF fb = {};   // sample i-1 (valid when fb_step == i-1)
         int64_t fb_step = -1;
         float Gc[3] = {0.0f, 0.0f, 0.0f}, guc = 0.0f;   // carry: sample i-1 so far
         bool nzc = false;
         float4 pb = make_float4(0.f, 0.f, 0.f, 0.f), pa = pb;   // sample i-1
-        int64_t J = 0;   // sample i-1 at J + f
+        int J = 0;   // sample i-1 at J + f
         // the pixel's record-gradient rows are read in increasing j: with n_bins a multiple
         // of 4 (16-byte aligned rows) a lane keeps the 16-byte chunk of each row holding the
         // current j, one vector load per row and 4 bins instead of one scalar per bin (the
         // lanes of a warp read 32 different rows, so loads cost one L1 wavefront per lane)
-        int64_t jc = -4;
+        int jc = -4;
         float4 c0 = make_float4(0.f, 0.f, 0.f, 0.f), c1 = c0, c2 = c0;
         float f = 0.0f;
         for (int64_t i0 = 0; i0 < p.ns1; i0 += kAdjTile) {
@@ -599,7 +594,7 @@ __global__ void __launch_bounds__(kAdjThreads) adj_deposit_mixed_kernel(AdjArgs 
             }
             __syncthreads();
             // sample i0 with the FP64 adjoint's expression: J0 + f0
-            int64_t J0;
+            int J0;
             float f0;
             exact_coord(u_fp64(s_anc[0], s_anc[1], s_anc[2], s_anc[3]), J0, f0);
             for (int q = 0; q < n; ++q) {
@@ -609,7 +604,7 @@ __global__ void __launch_bounds__(kAdjThreads) adj_deposit_mixed_kernel(AdjArgs 
                 // advanced from sample i-1 by the step's FP32 increment, and recomputed in
                 // FP64 when the fraction lies within kAdjGuard of an integer, so that the
                 // floors -- which grid points a step holds -- are those of the FP64 adjoint
-                int64_t Ji;
+                int Ji;
                 float fi;
                 if (q == 0) {
                     Ji = J0;
@@ -619,82 +614,77 @@ __global__ void __launch_bounds__(kAdjThreads) adj_deposit_mixed_kernel(AdjArgs 
                     float u = f + fmaf(wz32, d.w, fmaf(wy32, d.z, fmaf(wx32, d.y, s32 * d.x)));
                     u = fminf(fmaxf(u, -1.0e9f), 1.0e9f);
                     const float fl = floorf(u);
-                    Ji = J + (int64_t)fl;
+                    Ji = min(max(J + (int)fl, -1000000000), 1000000000);
                     fi = u - fl;
-                    if (fi < kAdjGuard || fi > 1.0f - kAdjGuard) {
+                    if (fi < kAdjGuard || fi > 1.0f - kAdjGuard || abs(J) > 900000000 ||
+                        abs(Ji) > 900000000) {   // (a clamped coordinate is no start to add to)
                         const double* rq = rk + 3 * i;
                         exact_coord(u_fp64(tk[i], rq[0], rq[1], rq[2]), Ji, fi);
                     }
                 }
                 // the step (i-1, i] relative to Jf = J_(i-1): ub = f_(i-1), ua = u_i - Jf
-                const int64_t Jf = J, dJ = Ji - J;
+                const int dJ = Ji - J;
                 const float ub = f;
                 const float ua = (dJ > -(1 << 24) && dJ < (1 << 24)) ? (float)dJ + fi : 1.0e9f;
                 float Gn[3] = {0.0f, 0.0f, 0.0f}, gun = 0.0f;   // contributions to sample i
-                bool nzn = false;
-                if (i > 0 && active) {
-                    int64_t ja = J + 1, jz = Ji;
-                    if (ja < 0) ja = 0;
-                    if (jz > p.n_bins - 1) jz = p.n_bins - 1;
-                    if (ja <= jz) {
-                        if (fb_step != i - 1) field_acc_f32(nf, pb, pa, Fb);
-                        float Fa[3];
-                        field_acc_f32(nf, cb, ca, Fa);
-                        const float iden = __fdividef(1.0f, ua - ub);
-                        const float d0 = Fa[0] - Fb[0], d1 = Fa[1] - Fb[1], d2 = Fa[2] - Fb[2];
-                        for (int64_t j = ja; j <= jz; ++j) {
-                            const float tj = (float)(j - Jf);
-                            const float wa = (ua - tj) * iden, wb = (tj - ub) * iden;
-                            float R0, R1, R2;
-                            if (vec) {   // 16-byte chunks of the three rows, reloaded per 4 bins
-                                if ((j & ~int64_t(3)) != jc) {
-                                    jc = j & ~int64_t(3);
-                                    c0 = __ldg(reinterpret_cast<const float4*>(R + jc));
-                                    c1 = __ldg(reinterpret_cast<const float4*>(R + p.n_bins + jc));
-                                    c2 = __ldg(reinterpret_cast<const float4*>(R + 2 * p.n_bins + jc));
-                                }
-                                const int e = (int)(j & 3);
-                                R0 = e == 0 ? c0.x : e == 1 ? c0.y : e == 2 ? c0.z : c0.w;
-                                R1 = e == 0 ? c1.x : e == 1 ? c1.y : e == 2 ? c1.z : c1.w;
-                                R2 = e == 0 ? c2.x : e == 1 ? c2.y : e == 2 ? c2.z : c2.w;
-                            } else {
-                                R0 = R[j];
-                                R1 = R[p.n_bins + j];
-                                R2 = R[2 * p.n_bins + j];
+                SampleF fa;
+                const int ja = max(J + 1, 0), jz = min(Ji, nb1);
+                const bool step = i > 0 && active && ja <= jz;   // the step holds grid points
+                if (step) {
+                    if (fb_step != i - 1) sample_field_f32(nf, pb, pa, fb);
+                    sample_field_f32(nf, cb, ca, fa);
+                    const float iden = __fdividef(1.0f, ua - ub);
+                    const float d0 = fa.F[0] - fb.F[0], d1 = fa.F[1] - fb.F[1],
+                                d2 = fa.F[2] - fb.F[2];
+                    float tj = (float)(ja - J);
+                    for (int j = ja; j <= jz; ++j, tj += 1.0f) {
+                        const float wa = (ua - tj) * iden, wb = (tj - ub) * iden;
+                        float R0, R1, R2;
+                        if (vec) {   // 16-byte chunks of the three rows, reloaded per 4 bins
+                            if ((j & ~3) != jc) {
+                                jc = j & ~3;
+                                c0 = __ldg(reinterpret_cast<const float4*>(R + jc));
+                                c1 = __ldg(reinterpret_cast<const float4*>(R + p.n_bins + jc));
+                                c2 = __ldg(reinterpret_cast<const float4*>(R + 2 * p.n_bins + jc));
                             }
-                            Gc[0] = fmaf(R0, wa, Gc[0]);
-                            Gc[1] = fmaf(R1, wa, Gc[1]);
-                            Gc[2] = fmaf(R2, wa, Gc[2]);
-                            Gn[0] = fmaf(R0, wb, Gn[0]);
-                            Gn[1] = fmaf(R1, wb, Gn[1]);
-                            Gn[2] = fmaf(R2, wb, Gn[2]);
-                            const float dw = fmaf(R2, d2, fmaf(R1, d1, R0 * d0)) * iden;
-                            gun = fmaf(-dw, wb, gun);
-                            guc = fmaf(-dw, wa, guc);
+                            const int e = j & 3;
+                            R0 = e == 0 ? c0.x : e == 1 ? c0.y : e == 2 ? c0.z : c0.w;
+                            R1 = e == 0 ? c1.x : e == 1 ? c1.y : e == 2 ? c1.z : c1.w;
+                            R2 = e == 0 ? c2.x : e == 1 ? c2.y : e == 2 ? c2.z : c2.w;
+                        } else {
+                            R0 = R[j];
+                            R1 = R[p.n_bins + j];
+                            R2 = R[2 * p.n_bins + j];
                         }
-                        nzc = true;
-                        nzn = true;
-                        Fb[0] = Fa[0];
-                        Fb[1] = Fa[1];
-                        Fb[2] = Fa[2];
-                        fb_step = i;
+                        Gc[0] = fmaf(R0, wa, Gc[0]);
+                        Gc[1] = fmaf(R1, wa, Gc[1]);
+                        Gc[2] = fmaf(R2, wa, Gc[2]);
+                        Gn[0] = fmaf(R0, wb, Gn[0]);
+                        Gn[1] = fmaf(R1, wb, Gn[1]);
+                        Gn[2] = fmaf(R2, wb, Gn[2]);
+                        const float dw = fmaf(R2, d2, fmaf(R1, d1, R0 * d0)) * iden;
+                        gun = fmaf(-dw, wb, gun);
+                        guc = fmaf(-dw, wa, guc);
                     }
                 }
                 if (i > 0)
-                    flush_sample_f32(p, active, nf, k, i - 1, pb, pa, Gc, guc, nzc, r_scale,
-                                     u_scale);
+                    flush_sample_f32(p, nf, k * p.ns1 + i - 1, fb, pa, Gc, guc, nzc || step);
                 Gc[0] = Gn[0];
                 Gc[1] = Gn[1];
                 Gc[2] = Gn[2];
                 guc = gun;
-                nzc = nzn;
+                nzc = step;
+                if (step) {
+                    fb = fa;
+                    fb_step = i;
+                }
                 J = Ji;
                 f = fi;
                 pb = cb;
                 pa = ca;
             }
         }
-        flush_sample_f32(p, active, nf, k, p.ns1 - 1, pb, pa, Gc, guc, nzc, r_scale, u_scale);
+        flush_sample_f32(p, nf, k * p.ns1 + p.ns1 - 1, fb, pa, Gc, guc, nzc);
     }
 }
 
