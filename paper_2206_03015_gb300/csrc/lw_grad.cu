@@ -372,11 +372,11 @@ __global__ void __launch_bounds__(kAdjThreads) adj_deposit_kernel(AdjArgs p) {
 
 // ------------------------------------------------------------ mixed-precision adjoint
 //
-// (2,048 electrons x 4,096 steps x 1,024 pixels x 16,384 bins: 269 ms with 64-bit grid indices,
-// whose conversions held the FP64 pipe at 71 %, a second field evaluation in the chain rule and
-// 45 shuffles per sample; 32-bit indices, one evaluation and warp_sum9 take 197 ms.  What
-// remains is latency: 54 % of the issue slots at 5 warps per scheduler, long scoreboard on the
-// record gradient's rows.)
+// Bound by issue and latency.  2,048 electrons x 4,096 steps x 1,024 pixels x 16,384 bins: 269 ms
+// with 64-bit grid indices (their conversions held the FP64 pipe at 71 %), a second field
+// evaluation in the chain rule and 45 shuffles per sample; 197 ms with 32-bit indices, one
+// evaluation and warp_sum9; 152 ms with FP32 constants that are not converted again per step and
+// the exact coordinate out of line, so that seven CTAs per SM are resident instead of four.
 //
 // The same transpose in mixed precision: the bin coordinate of each tile's first sample in
 // FP64 and, within the tile of 64 samples, each sample's as an integer plus an FP32
@@ -411,14 +411,31 @@ __device__ __forceinline__ int adj_exponent(unsigned long long mx) {
     return (mx == 0 || e > 1000 || e < -1000) ? 0 : e;
 }
 
-__global__ void adj_to_f32_kernel(const double* __restrict__ R, int64_t n,
+// dL/drec scaled and rounded to FP32.  With n_bins a multiple of 4 a pixel's three rows are
+// interleaved in groups of four bins (x, y, z of bins 4 q .. 4 q + 3: 48 bytes), so that the lanes
+// of a warp, each walking its own pixel, keep one cache line in use instead of three: the
+// adjoint's L1 working set is what limits its resident warps.
+__global__ void adj_to_f32_kernel(const double* __restrict__ R, int64_t n_pix, int64_t n_bins,
                                   const unsigned long long* __restrict__ mx,
                                   float* __restrict__ Rf, double* __restrict__ rscale) {
     const int e = adj_exponent(*mx);
     const double down = ldexp(1.0, -e);
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        Rf[i] = (float)(R[i] * down);
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if ((n_bins & 3) == 0) {
+        const int64_t per = n_bins / 4;
+        for (int64_t g = i0; g < n_pix * per; g += step) {
+            const int64_t m = g / per, q = g - m * per;
+            for (int c = 0; c < 3; ++c) {
+                const double* r = R + (3 * m + c) * n_bins + 4 * q;
+                reinterpret_cast<float4*>(Rf)[3 * g + c] =
+                    make_float4((float)(r[0] * down), (float)(r[1] * down), (float)(r[2] * down),
+                                (float)(r[3] * down));
+            }
+        }
+    } else {
+        for (int64_t i = i0; i < 3 * n_pix * n_bins; i += step) Rf[i] = (float)(R[i] * down);
+    }
     if (blockIdx.x == 0 && threadIdx.x == 0) *rscale = ldexp(1.0, e);
 }
 
@@ -502,48 +519,53 @@ __global__ void adj_finish_kernel(const float* __restrict__ f, int64_t n_samples
 // ulps of the step's terms).
 constexpr float kAdjGuard = 1.0f / (1 << 12);
 
-__global__ void __launch_bounds__(kAdjThreads) adj_deposit_mixed_kernel(AdjArgs p) {
+// The FP64 adjoint's bin coordinate of a sample (t, x) for the direction n, as floor + FP32
+// fraction.  32-bit: conversions from and to 64-bit integers run on the FP64 pipe; coordinates are
+// clamped to +-1e9, far beyond any grid.  Out of line, reading its direction again: inlined it
+// keeps doubles in registers throughout.
+__device__ __noinline__ int2 adj_exact_coord(const double* n, const double* x, double t,
+                                             double t_min, double inv_dtu) {
+    double u = __dmul_rn(__dsub_rn(advanced_time_fp64(n[0], n[1], n[2], x[0], x[1], x[2], t), t_min),
+                         inv_dtu);
+    u = fmin(fmax(u, -1.0e9), 1.0e9);
+    const double fl = floor(u);
+    return make_int2((int)fl, __float_as_int((float)(u - fl)));
+}
+
+__global__ void __launch_bounds__(kAdjThreads, 7) adj_deposit_mixed_kernel(AdjArgs p) {
     // one tile of samples i0 .. i0 + kAdjTile - 1, staged once per CTA: each sample's step
     // from the previous one (FP64 differences rounded to FP32) and its fields' inputs
     __shared__ float4 s_d[kAdjTile];   // (tau_i - tau_i-1, r_i - r_i-1), tau = t - z/c0
-    __shared__ float4 s_b[kAdjTile];   // (beta_x, beta_y, 1 - beta_z, |beta| < 1)
-    __shared__ float4 s_a[kAdjTile];   // (beta_dot, 0)
-    __shared__ double s_anc[4];        // (t, r) of sample i0
+    // (slot q + 1: sample i0 + q, slot 0: the sample before the tile)
+    __shared__ float4 s_b[kAdjTile + 1];   // (beta_x, beta_y, 1 - beta_z, |beta| < 1)
+    __shared__ float4 s_a[kAdjTile + 1];   // (beta_dot, 0)
     const int64_t m = (int64_t)blockIdx.x * kAdjThreads + threadIdx.x;
     const bool active = m < p.n_pix;
-    double nx = 0.0, ny = 0.0, nz = 1.0;
-    if (active) {
-        nx = p.n_hat[3 * m];
-        ny = p.n_hat[3 * m + 1];
-        nz = p.n_hat[3 * m + 2];
-    }
+    const double* n_hat = p.n_hat + (active ? 3 * m : 0);   // inactive lanes follow pixel 0
     NF nf;
-    nf.x = (float)nx;
-    nf.y = (float)ny;
-    nf.z = (float)nz;
-    nf.omz = (float)(1.0 - nz);
-    // bin coordinate u = (t_a - t_min)/dt_u = (tau - t_min)/dt_u + w . r with the pixel's
-    // slope w = (-n_x, -n_y, 1 - n_z) / (c0 dt_u): in FP64 at each tile's first sample; from
-    // there on as J + f (integer, FP32 fraction) advanced by each step's FP32 increment
-    // s dtau + w . dr, so that the weights see small numbers
-    const double sw = kInvC0 * p.inv_dtu;
-    const double wx = -nx * sw, wy = -ny * sw, wz = (1.0 - nz) * sw;
-    const float s32 = (float)p.inv_dtu, wx32 = (float)wx, wy32 = (float)wy, wz32 = (float)wz;
+    float s32, wx32, wy32, wz32;
+    {
+        const double nx = n_hat[0], ny = n_hat[1], nz = n_hat[2];
+        nf.x = (float)nx;
+        nf.y = (float)ny;
+        nf.z = (float)nz;
+        nf.omz = (float)(1.0 - nz);
+        // bin coordinate u = (t_a - t_min)/dt_u = (tau - t_min)/dt_u + w . r with the pixel's slope
+        // w = (-n_x, -n_y, 1 - n_z) / (c0 dt_u): in FP64 at each tile's first sample; from there on
+        // as J + f (integer, FP32 fraction) advanced by each step's FP32 increment s dtau + w . dr,
+        // so that the weights see small numbers
+        const double sw = kInvC0 * p.inv_dtu;
+        s32 = (float)p.inv_dtu;
+        wx32 = (float)(-nx * sw);
+        wy32 = (float)(-ny * sw);
+        wz32 = (float)((1.0 - nz) * sw);
+    }
+    // the rounded values are made opaque: the compiler otherwise converts the doubles again in
+    // every step to save registers (FP64 pipe 71-80 % busy at 96 registers)
+    asm volatile("" : "+f"(s32), "+f"(wx32), "+f"(wy32), "+f"(wz32));
+    asm volatile("" : "+f"(nf.x), "+f"(nf.y), "+f"(nf.z), "+f"(nf.omz));
     const float* R = p.dLdrec_f + (active ? m * 3 * p.n_bins : 0);
     const bool vec = (p.n_bins & 3) == 0;
-    // the FP64 adjoint's bin coordinate of a sample, and its split into floor + fraction
-    auto u_fp64 = [&](double t, double x, double y, double z) {
-        return __dmul_rn(__dsub_rn(advanced_time_fp64(nx, ny, nz, x, y, z, t), p.t_min),
-                         p.inv_dtu);
-    };
-    // (32-bit integers: conversions from and to 64-bit ones run on the FP64 pipe, which ten of
-    // them per sample kept 71 % busy; coordinates are clamped to +-1e9, far beyond any grid)
-    auto exact_coord = [&](double u, int& Jo, float& fo) {
-        u = fmin(fmax(u, -1.0e9), 1.0e9);
-        const double fl = floor(u);
-        Jo = (int)fl;
-        fo = (float)(u - fl);
-    };
     const int nb1 = (int)p.n_bins - 1;
     const int64_t k0 = (int64_t)blockIdx.y * p.e_chunk;
     const int64_t k1 = min(k0 + p.e_chunk, p.n_e);
@@ -556,24 +578,23 @@ __global__ void __launch_bounds__(kAdjThreads) adj_deposit_mixed_kernel(AdjArgs 
         int64_t fb_step = -1;
         float Gc[3] = {0.0f, 0.0f, 0.0f}, guc = 0.0f;   // carry: sample i-1 so far
         bool nzc = false;
-        float4 pb = make_float4(0.f, 0.f, 0.f, 0.f), pa = pb;   // sample i-1
         int J = 0;   // sample i-1 at J + f
-        // the pixel's record-gradient rows are read in increasing j: with n_bins a multiple
-        // of 4 (16-byte aligned rows) a lane keeps the 16-byte chunk of each row holding the
-        // current j, one vector load per row and 4 bins instead of one scalar per bin (the
-        // lanes of a warp read 32 different rows, so loads cost one L1 wavefront per lane)
+        // the record gradient is read in increasing j: with n_bins a multiple of 4 a lane keeps
+        // the group of four bins holding the current j, three vector loads per group instead
+        // of three scalars per bin (the lanes of a warp read 32 different pixels, so loads
+        // cost one L1 wavefront per lane)
         int jc = -4;
         float4 c0 = make_float4(0.f, 0.f, 0.f, 0.f), c1 = c0, c2 = c0;
         float f = 0.0f;
         for (int64_t i0 = 0; i0 < p.ns1; i0 += kAdjTile) {
             const int n = (int)min((int64_t)kAdjTile, p.ns1 - i0);
             __syncthreads();
-            for (int q = threadIdx.x; q < n; q += kAdjThreads) {
+            for (int q = (i0 > 0 ? -1 : 0) + (int)threadIdx.x; q < n; q += kAdjThreads) {
                 const int64_t i = i0 + q;
                 const double* rq = rk + 3 * i;
                 const double* bq = bk + 3 * i;
                 const double* aq = ak + 3 * i;
-                if (i > 0) {
+                if (i > 0 && q >= 0) {
                     const double tau = tk[i] - rq[2] * kInvC0;
                     const double taup = tk[i - 1] - rq[-1] * kInvC0;
                     s_d[q] = make_float4((float)(tau - taup), (float)(rq[0] - rq[-3]),
@@ -582,45 +603,35 @@ __global__ void __launch_bounds__(kAdjThreads) adj_deposit_mixed_kernel(AdjArgs 
                 const double bb = __dadd_rn(__dadd_rn(__dmul_rn(bq[0], bq[0]),
                                                       __dmul_rn(bq[1], bq[1])),
                                             __dmul_rn(bq[2], bq[2]));
-                s_b[q] = make_float4((float)bq[0], (float)bq[1], (float)(1.0 - bq[2]),
+                s_b[q + 1] = make_float4((float)bq[0], (float)bq[1], (float)(1.0 - bq[2]),
                                      bb < 1.0 ? 1.0f : 0.0f);
-                s_a[q] = make_float4((float)aq[0], (float)aq[1], (float)aq[2], 0.0f);
-            }
-            if (threadIdx.x == 0) {
-                s_anc[0] = tk[i0];
-                s_anc[1] = rk[3 * i0];
-                s_anc[2] = rk[3 * i0 + 1];
-                s_anc[3] = rk[3 * i0 + 2];
+                s_a[q + 1] = make_float4((float)aq[0], (float)aq[1], (float)aq[2], 0.0f);
             }
             __syncthreads();
-            // sample i0 with the FP64 adjoint's expression: J0 + f0
-            int J0;
-            float f0;
-            exact_coord(u_fp64(s_anc[0], s_anc[1], s_anc[2], s_anc[3]), J0, f0);
             for (int q = 0; q < n; ++q) {
                 const int64_t i = i0 + q;
-                const float4 cb = s_b[q], ca = s_a[q];
                 // sample i at Ji + fi: the tile's first from the FP64 anchor, the others
                 // advanced from sample i-1 by the step's FP32 increment, and recomputed in
                 // FP64 when the fraction lies within kAdjGuard of an integer, so that the
                 // floors -- which grid points a step holds -- are those of the FP64 adjoint
                 int Ji;
                 float fi;
-                if (q == 0) {
-                    Ji = J0;
-                    fi = f0;
-                } else {
+                bool exact = q == 0;
+                if (!exact) {
                     const float4 d = s_d[q];
                     float u = f + fmaf(wz32, d.w, fmaf(wy32, d.z, fmaf(wx32, d.y, s32 * d.x)));
                     u = fminf(fmaxf(u, -1.0e9f), 1.0e9f);
                     const float fl = floorf(u);
                     Ji = min(max(J + (int)fl, -1000000000), 1000000000);
                     fi = u - fl;
-                    if (fi < kAdjGuard || fi > 1.0f - kAdjGuard || abs(J) > 900000000 ||
-                        abs(Ji) > 900000000) {   // (a clamped coordinate is no start to add to)
-                        const double* rq = rk + 3 * i;
-                        exact_coord(u_fp64(tk[i], rq[0], rq[1], rq[2]), Ji, fi);
-                    }
+                    // (a clamped coordinate is no start to add to)
+                    exact = fi < kAdjGuard || fi > 1.0f - kAdjGuard || abs(J) > 900000000 ||
+                            abs(Ji) > 900000000;
+                }
+                if (exact) {
+                    const int2 e = adj_exact_coord(n_hat, rk + 3 * i, tk[i], p.t_min, p.inv_dtu);
+                    Ji = e.x;
+                    fi = __int_as_float(e.y);
                 }
                 // the step (i-1, i] relative to Jf = J_(i-1): ub = f_(i-1), ua = u_i - Jf
                 const int dJ = Ji - J;
@@ -631,8 +642,8 @@ __global__ void __launch_bounds__(kAdjThreads) adj_deposit_mixed_kernel(AdjArgs 
                 const int ja = max(J + 1, 0), jz = min(Ji, nb1);
                 const bool step = i > 0 && active && ja <= jz;   // the step holds grid points
                 if (step) {
-                    if (fb_step != i - 1) sample_field_f32(nf, pb, pa, fb);
-                    sample_field_f32(nf, cb, ca, fa);
+                    if (fb_step != i - 1) sample_field_f32(nf, s_b[q], s_a[q], fb);
+                    sample_field_f32(nf, s_b[q + 1], s_a[q + 1], fa);
                     const float iden = __fdividef(1.0f, ua - ub);
                     const float d0 = fa.F[0] - fb.F[0], d1 = fa.F[1] - fb.F[1],
                                 d2 = fa.F[2] - fb.F[2];
@@ -640,12 +651,13 @@ __global__ void __launch_bounds__(kAdjThreads) adj_deposit_mixed_kernel(AdjArgs 
                     for (int j = ja; j <= jz; ++j, tj += 1.0f) {
                         const float wa = (ua - tj) * iden, wb = (tj - ub) * iden;
                         float R0, R1, R2;
-                        if (vec) {   // 16-byte chunks of the three rows, reloaded per 4 bins
+                        if (vec) {   // a group of four bins of the three rows, reloaded when left
                             if ((j & ~3) != jc) {
                                 jc = j & ~3;
-                                c0 = __ldg(reinterpret_cast<const float4*>(R + jc));
-                                c1 = __ldg(reinterpret_cast<const float4*>(R + p.n_bins + jc));
-                                c2 = __ldg(reinterpret_cast<const float4*>(R + 2 * p.n_bins + jc));
+                                const float4* g = reinterpret_cast<const float4*>(R + 3 * jc);
+                                c0 = __ldg(g);
+                                c1 = __ldg(g + 1);
+                                c2 = __ldg(g + 2);
                             }
                             const int e = j & 3;
                             R0 = e == 0 ? c0.x : e == 1 ? c0.y : e == 2 ? c0.z : c0.w;
@@ -668,7 +680,7 @@ __global__ void __launch_bounds__(kAdjThreads) adj_deposit_mixed_kernel(AdjArgs 
                     }
                 }
                 if (i > 0)
-                    flush_sample_f32(p, nf, k * p.ns1 + i - 1, fb, pa, Gc, guc, nzc || step);
+                    flush_sample_f32(p, nf, k * p.ns1 + i - 1, fb, s_a[q], Gc, guc, nzc || step);
                 Gc[0] = Gn[0];
                 Gc[1] = Gn[1];
                 Gc[2] = Gn[2];
@@ -680,16 +692,14 @@ __global__ void __launch_bounds__(kAdjThreads) adj_deposit_mixed_kernel(AdjArgs 
                 }
                 J = Ji;
                 f = fi;
-                pb = cb;
-                pa = ca;
             }
         }
-        flush_sample_f32(p, nf, k * p.ns1 + p.ns1 - 1, fb, pa, Gc, guc, nzc);
+        flush_sample_f32(p, nf, k * p.ns1 + p.ns1 - 1, fb, s_a[(p.ns1 - 1) % kAdjTile + 1], Gc, guc, nzc);
     }
 }
 
 int pick_chunk(int64_t n_e, int64_t tiles) {
-    const int64_t target = (int64_t)kSms * 16;
+    const int64_t target = (int64_t)kSms * 64;
     int64_t chunk = (n_e * tiles + target - 1) / target;
     if (chunk < 1) chunk = 1;
     if (chunk > n_e) chunk = n_e;
@@ -819,7 +829,7 @@ extern "C" int lw_spectrum_grad(const lw_traj* traj, const lw_detector* det, con
     const int64_t n_rec = rows * N;
     const int rg = (int)std::min<int64_t>((n_rec + 255) / 256, (int64_t)kSms * 8);
     adj_absmax_kernel<<<rg, 256, 0, st>>>(dLdrec, n_rec, mx);
-    adj_to_f32_kernel<<<rg, 256, 0, st>>>(dLdrec, n_rec, mx, Rf, rscale);
+    adj_to_f32_kernel<<<rg, 256, 0, st>>>(dLdrec, det->n_pix, N, mx, Rf, rscale);
     if (launch_status() != LW_OK) return LW_ECUDA;
     a.dLdrec_f = Rf;
     a.rscale = rscale;

@@ -42,3 +42,24 @@ def test_fp64_adjoint_against_oracle(n_e, n_s, n_pix, bins, lo_f, hi_f):
         # as the element-wise bound of the other adjoint tests: D = 1 - n.beta carries 1e-16 in
         # 1e-3, the record's transforms and their products a few more
         assert np.abs(a.cpu().numpy() - b).max() <= 1e-9 * np.abs(b).max()
+
+
+@pytest.mark.parametrize("n_e,n_s,n_pix,bins,lo_f,hi_f", [
+    (1, 1, 1, 2, -0.01, 1.01), (2, 63, 3, 16, -0.01, 1.01), (1, 64, 33, 256, -0.01, 1.01),
+    (3, 65, 5, 64, -0.01, 1.01), (1, 128, 129, 32, -0.01, 1.01), (1, 200, 31, 512, 0.4, 0.6),
+    (2, 150, 7, 64, -1.0, 0.5), (1, 130, 2, 4096, -0.01, 1.01)])
+def test_mixed_adjoint_against_fp64(n_e, n_s, n_pix, bins, lo_f, hi_f):
+    """The mixed adjoint at its own cuts (tiles of 64 samples with the sample before, groups of four
+    bins, the last sample) against the FP64 adjoint of the same X', element by element."""
+    tr, n_hat, grid = _case(n_e, n_s, n_pix, bins, lo_f, hi_f)
+    g = np.random.Generator(np.random.PCG64(2)).standard_normal((n_pix, bins // 2 + 1))
+    g = torch.from_numpy(g).cuda()
+    traj = lw.lw_trajectories_upload(tr.t, tr.r, tr.beta, tr.beta_dot)
+    det = lw.Detector(n_hat)
+    rec = lw.lw_deposit_time_domain(traj, det, grid, lw.LW_FP64)
+    _, X = lw.lw_spectrum(rec, lw.LW_FP64, n_pix, grid, want_X=True)
+    want = lw.lw_spectrum_grad(traj, det, grid, X, g)
+    got = lw.lw_spectrum_grad(traj, det, grid, X.to(torch.complex64), g)
+    for a, b in zip(got, want):
+        # the bound of the mixed adjoint's comparison with the oracle
+        assert float((a - b).abs().max()) <= 1e-4 * float(b.abs().max())
