@@ -66,6 +66,7 @@ struct DepositArgs {
     void* record;
     int32_t* status;
     int e_chunk;
+    const double* span;   // mixed: mean advance, or null where no tile can be dense (walk_tile)
 };
 
 // ------------------------------------------------------------------ FP64
@@ -590,6 +591,111 @@ __device__ __forceinline__ float fd_rel(const PixelConst& pc, float4 f4, float2 
 // floor(I + f) - I for a double-FP32 fraction f that lies within rounding of [0, 1)
 __device__ __forceinline__ int frac_floor(float f) { return f >= 1.0f ? 1 : (f < 0.0f ? -1 : 0); }
 
+// Walk of one warp over a staged block whose grid points are dense: instead of locating every grid
+// point by a search (about 230 instructions each), the block's samples are evaluated once per
+// pixel, 32 at a time -- coordinate, last grid point at or before it and field, one sample per
+// lane -- and the grid points between consecutive samples are then taken one per lane, in order,
+// so that the record updates of a warp are consecutive grid points of one pixel.  A grid point
+// belongs to the same step as in the search (the first sample whose coordinate reaches it; the
+// run's bounds ja .. ja + K - 1 go to the first and the last step).
+// The samples of a segment cost about 90 instructions per pixel whatever their grid points, and a
+// round of 32 grid points about 18, against 32 x 7.2 by search: the walk is the cheaper one above
+// kWalkDensity grid points per step.  2,048 co-located electrons x 4,096 steps x 1,024 pixels x
+// 16,384 bins (1 to 5 grid points per step): 238 ms by search, 82 ms walked.
+constexpr double kWalkDensity = 0.45;
+constexpr int kWalkTile = 512;  // pixels that share a decision
+constexpr int kWalkMap = 256;   // grid points of a segment mapped to steps at a time
+
+template <int PIX, int ACC, int FL>
+__device__ __forceinline__ void walk_block(const float4* s_scan, const float4* s_f4,
+                                        const float2* s_f2, int ns, const float4* s_wh,
+                                        const int4* s_job, int2 K2, int2 JA2, float s32,
+                                        float inv_sc, float c0_over_R, int64_t n_bins,
+                                        unsigned char* tile_rec, float4* stage,
+                                        unsigned char* map) {
+    const int lane = threadIdx.x & 31;
+    const uint64_t row_bytes =
+        4ull * (ACC == kAccF32X4 ? 4 : ACC == kAccF32 ? 3 : 6) * (uint64_t)n_bins;
+    // stage[0]: the sample before the segment, stage[1 + l]: the segment's sample l, each
+    // (coordinate, field)
+    for (int slot = 0; slot < 32 * PIX; ++slot) {   // s_wh, s_job: the warp's slots
+        const int K = __shfl_sync(0xffffffffu, slot % PIX ? K2.y : K2.x, slot / PIX);
+        if (K == 0) continue;
+        const int ja = __shfl_sync(0xffffffffu, slot % PIX ? JA2.y : JA2.x, slot / PIX);
+        const int4 jb = s_job[slot];
+        const float4 w = s_wh[slot];
+        const float f = __int_as_float(jb.y), xe = __int_as_float(jb.z);
+        unsigned char* const row = tile_rec + (uint64_t)__float_as_uint(w.w) * row_bytes;
+        PixelConst pc;
+        pc.nx = -w.x * inv_sc;
+        pc.ny = -w.y * inv_sc;
+        pc.omnz = w.z * inv_sc;
+        pc.nz = 1.0f - pc.omnz;
+        const float2 nxy = make_float2(pc.nx, pc.ny);
+        const int lo = ja - 1 - jb.x, hi = lo + K;   // last grid point before and of the run
+        int Jc = lo;                                  // last grid point of the samples so far
+        for (int r0 = 0; r0 <= ns && Jc < hi; r0 += 32) {
+            const int r = r0 + lane;   // sample (0: the anchor)
+            const int rc = min(r, ns);
+            const float x = rc == 0 ? 0.0f : rc == ns ? xe : coord(w, s32, s_scan[rc]);
+            float2 txy;
+            float tz, sc;
+            end_terms<FL>(pc, nxy, s_f4[rc], s_f2[rc], c0_over_R, 1.0f, txy, tz, sc);
+            // last J with fl(J - f) <= x
+            int J = (int)fminf(fmaxf(floorf(x + f), -1.0e9f), 1.0e9f);
+            if (__fsub_rn((float)(J + 1), f) <= x)
+                ++J;
+            else if (__fsub_rn((float)J, f) > x)
+                --J;
+            J = r == 0 ? lo : r >= ns ? hi : min(max(J, Jc), hi);
+            int before = __shfl_up_sync(0xffffffffu, J, 1);
+            if (lane == 0) before = Jc;
+            if (__any_sync(0xffffffffu, J < before)) {   // coordinates within rounding of one another
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) J = max(J, __shfl_up_sync(0xffffffffu, J, d));
+                before = __shfl_up_sync(0xffffffffu, J, 1);
+                if (lane == 0) before = Jc;
+            }
+            __syncwarp();   // the segment before is read
+            if (r0 > 0 && lane == 0) stage[0] = stage[32];
+            __syncwarp();
+            stage[1 + lane] = make_float4(x, txy.x * sc, txy.y * sc, tz * sc);
+            const int Je = __shfl_sync(0xffffffffu, J, 31);
+            for (int b0 = Jc; b0 < Je; b0 += kWalkMap) {   // grid points b0 + 1 .. b0 + kWalkMap
+                const int z = min(J - b0, kWalkMap);
+                for (int t = max(before - b0, 0); t < z; ++t) map[t] = (unsigned char)lane;
+                __syncwarp();
+                const int n = min(Je - b0, kWalkMap);
+                for (int t = lane; t < n; t += 32) {
+                    const int e = map[t];   // step from sample e - 1 to sample e of the segment
+                    const float4 a = stage[e], b = stage[e + 1];
+                    const int j = b0 + 1 + t;
+                    const float tJ = __fsub_rn((float)j, f);
+                    const float du = __fsub_rn(b.x, a.x);
+                    const float wb = du > 0.0f ? __fdividef(__fsub_rn(tJ, a.x), du) : 0.0f;
+                    deposit3_row<ACC>(row, j + jb.x, n_bins, fmaf(wb, b.y - a.y, a.y),
+                                      fmaf(wb, b.z - a.z, a.z), fmaf(wb, b.w - a.w, a.w));
+                }
+                __syncwarp();   // the map is rewritten
+            }
+            Jc = Je;
+        }
+        __syncwarp();
+    }
+}
+
+// Whether the electrons are walked for the 512 pixels around `pix`: the grid points per step that
+// the trajectories' mean advance (span, stored by the upload) gives the middle pixel.  Two launches
+// share a deposit's tiles by this test, so it is one function (out of line) of the call's arguments
+// only.  A test of every electron, by each of the search's CTAs, cost more than it sorted out
+// (36 FP64 instructions: 10 % of a 1,001-electron step).
+__device__ __noinline__ bool walk_tile(const double* span, const double* n_hat, int64_t n_pix,
+                                       int64_t pix, double steps, double inv_dtu) {
+    const double* n = n_hat + 3 * min(pix, n_pix - 1);
+    const double nr = (n[0] * span[1] + n[1] * span[2]) - (1.0 - n[2]) * span[3];
+    return (span[0] - nr * kInvC0) * inv_dtu > kWalkDensity * steps;
+}
+
 // The work of one CTA: pixel tile `tile` (kMixThreads * PIX pixels) and electron
 // chunk `chunk` (p.e_chunk electrons) of one variant.  Returns the status bits.
 //
@@ -621,9 +727,11 @@ __device__ __forceinline__ int frac_floor(float f) { return f >= 1.0f ? 1 : (f <
 // cluster over which the unit's sums are taken.  Without SPLIT
 // (one part, known at compile time) the deposit keeps the registers that the parts cost it
 // (80 instead of 74 with spills: 0.8 % of a 10,000-electron step).
-template <int PIX, int ACC, int FL, bool CHECK, bool SPLIT>
+enum { kSearch = 0, kWalk = 1, kCheck = 2 };   // deposit by search, by walk, or check
+template <int PIX, int ACC, int FL, int MODE, bool SPLIT>
 __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int64_t chunk,
                                          int part_ = 0, int parts_ = 1) {
+    constexpr bool CHECK = MODE == kCheck;
     const int part = SPLIT ? part_ : 0, parts = SPLIT ? parts_ : 1;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     constexpr int kSlots = kMixThreads * PIX;
@@ -637,7 +745,7 @@ __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int
     __shared__ int4 s_job[kSlots];                    // block: I, f, x_end
     __shared__ int s_ja[kSlots];                      // block: first grid point
     __shared__ int s_kp[kSlots];                      // block: job offset (lane-major)
-    __shared__ int2 s_tab[kWarpsMix][kJobTable];      // block: (slot, grid point) of job t
+    __shared__ __align__(16) int2 s_tab[kWarpsMix][kJobTable];   // block: (slot, grid point) of job t
     __shared__ __align__(8) uint64_t s_full[kMixStages];   // stage filled (bytes arrived)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -900,6 +1008,16 @@ __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int
                 tot += K[q];
                 Is[q] = Ie;
                 fs[q] = fe;
+            }
+            if constexpr (MODE == kWalk) {
+                for (int q = 0; q < PIX; ++q) K[q] += big[q];
+                __syncwarp();   // the warp's slot records are written
+                walk_block<PIX, ACC, FL>(
+                    s_scan, s_f4, s_f2, ns, s_wh + wslot, s_job + wslot,
+                    make_int2(K[0], K[PIX - 1]), make_int2(JA[0], JA[PIX - 1]), s32, inv_sc,
+                    c0_over_R, p.n_bins, tile_rec, reinterpret_cast<float4*>(&s_tab[warp][0]),
+                    reinterpret_cast<unsigned char*>(&s_tab[warp][kJobTable / 2 + 4]));
+                continue;
             }
             // Grid point j (absolute) of slot sl with block data I, f, xe (coordinate of the
             // block's last sample relative to the anchor) and slope w: its step ends at the
@@ -1298,13 +1416,33 @@ __global__ void __launch_bounds__(kFp64Threads) deposit_fp64_kernel(DepositArgs 
     block_status_or(p.status, bits);
 }
 
+// walk_tile for the CTA (thread 0 decides)
+__device__ __forceinline__ bool tile_is_dense(const DepositArgs& p, int64_t pix0) {
+    int dense = 0;
+    if (threadIdx.x == 0)
+        dense = walk_tile(p.span, p.n_hat, p.n_pix, pix0 / kWalkTile * kWalkTile + kWalkTile / 2,
+                          (double)(p.ns1 - 1), p.inv_dtu);
+    return __syncthreads_or(dense) != 0;
+}
+
 template <int PIX, int ACC, int FL, bool SPLIT>
 __global__ void __launch_bounds__(kMixThreads, kMixMinBlocks) deposit_mixed_kernel(DepositArgs p) {
     // the precision check launched after this grid (programmatic dependent launch) may
     // start once every CTA of this grid has started: it fills the SMs of the last wave
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (p.span && tile_is_dense(p, (int64_t)blockIdx.x * (kMixThreads * PIX))) return;
     const int bits =
-        mixed_cta<PIX, ACC, FL, false, SPLIT>(p, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.z);
+        mixed_cta<PIX, ACC, FL, kSearch, SPLIT>(p, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.z);
+    block_status_or(p.status, bits);
+}
+
+// The tiles whose grid points are dense, walked (launched before the search; a launch without dense
+// tiles is about four waves of CTAs that end at once, 5 us).
+template <int ACC, int FL>
+__global__ void __launch_bounds__(kMixThreads, kMixMinBlocks) deposit_walk_kernel(DepositArgs p) {
+    if (!tile_is_dense(p, (int64_t)blockIdx.x * kMixThreads)) return;
+    const int bits = mixed_cta<1, ACC, FL, kWalk, true>(p, blockIdx.x, blockIdx.y, blockIdx.z,
+                                                        gridDim.z);
     block_status_or(p.status, bits);
 }
 
@@ -1319,7 +1457,7 @@ __global__ void __launch_bounds__(kMixThreads, kMixMinBlocks) deposit_mixed_kern
 template <int PIX, int FL>
 __global__ void __launch_bounds__(kMixThreads, kMixMinBlocks)
     deposit_check_kernel(DepositArgs p, int stride) {
-    const int bits = mixed_cta<PIX, kAccF32X4, FL, true, true>(p, blockIdx.x, (int64_t)blockIdx.y * stride,
+    const int bits = mixed_cta<PIX, kAccF32X4, FL, kCheck, true>(p, blockIdx.x, (int64_t)blockIdx.y * stride,
                                                           blockIdx.z, gridDim.z);
     block_status_or(p.status, bits & LW_ST_PRECISION);
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1351,7 +1489,7 @@ __global__ void __launch_bounds__(kMixThreads, kMixMinBlocks)
         if (u >= n_units) break;
         const BatchUnit un = units[u];
         const DepositArgs& p = c_batch_vars[un.variant];
-        const int bits = mixed_cta<PIX, ACC, FL, false, false>(p, un.tile, un.chunk);
+        const int bits = mixed_cta<PIX, ACC, FL, kSearch, false>(p, un.tile, un.chunk);
         block_status_or(p.status, bits);
     }
 }
@@ -1364,7 +1502,7 @@ __global__ void __launch_bounds__(kMixThreads, kMixMinBlocks)
     const BatchUnit un = units[u];
     const DepositArgs& p = c_batch_vars[un.variant];
     const int bits =
-        mixed_cta<PIX, kAccF32X4, FL, true, true>(p, un.tile, un.chunk, blockIdx.z, gridDim.z);
+        mixed_cta<PIX, kAccF32X4, FL, kCheck, true>(p, un.tile, un.chunk, blockIdx.z, gridDim.z);
     block_status_or(p.status, bits & LW_ST_PRECISION);
 }
 
@@ -1409,6 +1547,16 @@ BatchedKernel batched_kernel_fl(uint32_t fl) {
     return fl == 1 ? deposit_batched_kernel<kMixPix, ACC, 1>
            : fl == 2 ? deposit_batched_kernel<kMixPix, ACC, 2>
                      : deposit_batched_kernel<kMixPix, ACC, 3>;
+}
+template <int ACC>
+MixedKernel walk_kernel_fl(uint32_t fl) {
+    return fl == 1 ? deposit_walk_kernel<ACC, 1>
+           : fl == 2 ? deposit_walk_kernel<ACC, 2> : deposit_walk_kernel<ACC, 3>;
+}
+MixedKernel walk_kernel(int acc, uint32_t fl) {
+    return acc == kAccKahan ? walk_kernel_fl<kAccKahan>(fl)
+           : acc == kAccF32 ? walk_kernel_fl<kAccF32>(fl)
+           : acc == kAccF32X4 ? walk_kernel_fl<kAccF32X4>(fl) : walk_kernel_fl<kAccF64>(fl);
 }
 using CheckKernel = void (*)(DepositArgs, int);
 template <int PIX>
@@ -1542,6 +1690,25 @@ extern "C" int lw_deposit_time_domain(const lw_traj* traj, const lw_detector* de
         g.z = (unsigned)std::min<int64_t>(std::min<int64_t>(nbs, 64), (two_waves + ctas - 1) / ctas);
     }
     const size_t smem = kMixStages * stage_bytes(traj->block);   // staging ring
+    // dense tiles (decided on the device, walk_tile) are walked by a launch of their own where the
+    // grid can hold that many points per step
+    if ((double)grid->n_bins > kWalkDensity * (double)traj->n_s) {
+        a.span = traj_span(traj);
+        DepositArgs w = a;
+        const int64_t wx = (det->n_pix + kMixThreads - 1) / kMixThreads;
+        const int64_t rows = std::max<int64_t>(1, 2 * two_waves / wx);
+        w.e_chunk = (int)std::max<int64_t>(std::max<int64_t>(traj->n_e / rows, 1),
+                                           (traj->n_e + 65534) / 65535);
+        const int64_t chunks = (traj->n_e + w.e_chunk - 1) / w.e_chunk;
+        const int64_t parts = std::min<int64_t>(std::min<int64_t>(nbs, 64),
+                                                (two_waves + wx * chunks - 1) / (wx * chunks));
+        const MixedKernel wk = walk_kernel(acc_of(precision), field_flags);
+        if (cudaFuncSetAttribute(wk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+            cudaSuccess)
+            return LW_ECUDA;
+        wk<<<dim3((unsigned)wx, (unsigned)chunks, (unsigned)parts), kMixThreads, smem, st>>>(w);
+        if (launch_status() != LW_OK) return LW_ECUDA;
+    }
     // static tables + double-buffered staging exceed the 48 KB default: opt in
     const MixedKernel kern = split ? mixed_kernel<true>(acc_of(precision), field_flags)
                                    : mixed_kernel<false>(acc_of(precision), field_flags);

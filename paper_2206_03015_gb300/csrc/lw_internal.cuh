@@ -33,6 +33,21 @@ inline int launch_status() {
 
 inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
+// Scratch of the upload's electron ordering, at the 256-byte boundary after the order itself:
+// two ordered keys, bucket counters, and the electrons' mean advance from first to last sample
+// (t - z/c0, x, y, z), which the mixed deposit reads.
+constexpr int kOrderBuckets = 4096;
+struct OrderScratch {
+    unsigned long long keys[2];
+    int32_t counts[kOrderBuckets];
+    double span[4];
+};
+inline const double* traj_span(const lw_traj* t) {
+    const char* order = reinterpret_cast<const char*>(t->order);
+    return reinterpret_cast<const OrderScratch*>(order + align256(sizeof(int32_t) * (size_t)t->n_e))
+        ->span;
+}
+
 __device__ __forceinline__ void status_or(int32_t* st, int bits) {
     if (st && bits) atomicOr(st, bits);
 }

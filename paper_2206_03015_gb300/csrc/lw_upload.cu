@@ -19,9 +19,6 @@
 namespace lw {
 namespace {
 
-// Buckets of the electron ordering (light-front time of the first sample).
-constexpr int kOrderBuckets = 4096;
-
 struct TrajLayout {
     size_t status = 0, ends = 0, t = 0, r = 0, beta = 0, beta_dot = 0, scan = 0, field = 0,
            anchor = 0, order = 0, order_tmp = 0;
@@ -60,8 +57,8 @@ TrajLayout make_layout(int64_t n_e, int64_t n_s, int t_per_e, int sections, int 
     }
     L.order = off;
     off = align256(off + sizeof(int32_t) * (size_t)n_e);
-    L.order_tmp = off;   // two ordered keys (range) + kOrderBuckets counters
-    off = align256(off + 2 * sizeof(unsigned long long) + sizeof(int32_t) * kOrderBuckets);
+    L.order_tmp = off;
+    off = align256(off + sizeof(OrderScratch));
     L.total = off;
     return L;
 }
@@ -248,23 +245,29 @@ __global__ void ends_kernel(const double* __restrict__ t, int t_per_e,
 __device__ __forceinline__ double first_tau(const double* e) { return e[0] - e[3] * kInvC0; }
 
 __global__ void order_range_kernel(const double* __restrict__ ends, int64_t n_e,
-                                   unsigned long long* keys) {
+                                   unsigned long long* keys, double* span) {
     double lo = INFINITY, hi = -INFINITY;
+    double adv[4] = {0.0, 0.0, 0.0, 0.0};   // first to last sample: t - z/c0, x, y, z
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n_e;
          k += (int64_t)gridDim.x * blockDim.x) {
         const double v = first_tau(ends + 8 * k);
         if (isfinite(v)) {
             lo = fmin(lo, v);
             hi = fmax(hi, v);
+            const double* e = ends + 8 * k;
+            adv[0] += first_tau(e + 4) - v;
+            for (int c = 1; c < 4; ++c) adv[c] += e[4 + c] - e[c];
         }
     }
     for (int o = 16; o > 0; o >>= 1) {
         lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
         hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        for (int c = 0; c < 4; ++c) adv[c] += __shfl_xor_sync(0xffffffffu, adv[c], o);
     }
     if ((threadIdx.x & 31) == 0) {
         atomicMin(&keys[0], ordered_key(lo));
         atomicMax(&keys[1], ordered_key(hi));
+        for (int c = 0; c < 4; ++c) atomicAdd(&span[c], adv[c] / (double)n_e);
     }
 }
 
@@ -460,13 +463,14 @@ extern "C" int lw_trajectories_upload(const lw_traj_in* in, int32_t sections, in
     if (launch_status() != LW_OK) return LW_ECUDA;
     {
         int32_t* order = reinterpret_cast<int32_t*>(base + L.order);
-        unsigned long long* keys = reinterpret_cast<unsigned long long*>(base + L.order_tmp);
-        int32_t* counts = reinterpret_cast<int32_t*>(keys + 2);
-        if (cudaMemsetAsync(counts, 0, sizeof(int32_t) * kOrderBuckets, st) != cudaSuccess)
+        OrderScratch* tmp = reinterpret_cast<OrderScratch*>(base + L.order_tmp);
+        unsigned long long* keys = tmp->keys;
+        int32_t* counts = tmp->counts;
+        if (cudaMemsetAsync(counts, 0, sizeof(tmp->counts) + sizeof(tmp->span), st) != cudaSuccess)
             return LW_ECUDA;
         bounds_init_kernel<<<1, 1, 0, st>>>(keys);
         const int ge = grid_for(in->n_e, threads);
-        order_range_kernel<<<ge, threads, 0, st>>>(ends, in->n_e, keys);
+        order_range_kernel<<<ge, threads, 0, st>>>(ends, in->n_e, keys, tmp->span);
         order_count_kernel<<<ge, threads, 0, st>>>(ends, in->n_e, keys, counts);
         order_scan_kernel<<<1, 1024, 0, st>>>(counts);
         order_scatter_kernel<<<ge, threads, 0, st>>>(ends, in->n_e, keys, counts, order);
