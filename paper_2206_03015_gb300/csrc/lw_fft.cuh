@@ -116,6 +116,31 @@ __device__ __forceinline__ C mul_root16(C x, int k) {
     }
 }
 
+// (u, x) -> (u + r x, u - r x), r = exp(2 pi i k / 16).  FP64: the odd eighth roots' products
+// r2 (x.x -+ x.y) are fused into the sums (6 instructions instead of 8; the FP64 pipe bounds
+// those transforms).  FP32 keeps product and sum apart: its results are compared bit by bit.
+template <typename C>
+__device__ __forceinline__ void butterfly16(C& u, C& x, int k) {
+    const C v = mul_root16(x, k);
+    x = csub(u, v);
+    u = cadd(u, v);
+}
+__device__ __forceinline__ void butterfly16(double2& u, double2& x, int k) {
+    if (k == 2 || k == 6) {   // (1 + i)/sqrt 2, (-1 + i)/sqrt 2
+        const double r2 = 0.70710678118654752440;
+        const double d = x.x - x.y, s = x.x + x.y;
+        const double re = k == 2 ? d : -s, im = k == 2 ? s : d;
+        x.x = fma(-r2, re, u.x);
+        x.y = fma(-r2, im, u.y);
+        u.x = fma(r2, re, u.x);
+        u.y = fma(r2, im, u.y);
+        return;
+    }
+    const double2 v = mul_root16(x, k);
+    x = csub(u, v);
+    u = cadd(u, v);
+}
+
 template <typename C, int CN, bool PAD, int R>
 __device__ __forceinline__ void fft_pass(C* buf, int L, int sh, int s, const C* __restrict__ tw,
                                          int N) {
@@ -143,10 +168,7 @@ __device__ __forceinline__ void fft_pass(C* buf, int L, int sh, int s, const C* 
             for (int m = 0; m < G; ++m) {
                 if (m & half) continue;
                 // root exp(2 pi i r / 2^(st+1)) = 16th root number r * 8 / half
-                const C v = mul_root16(x[m + half], (m & (half - 1)) * (8 >> st));
-                const C u = x[m];
-                x[m] = cadd(u, v);
-                x[m + half] = csub(u, v);
+                butterfly16(x[m], x[m + half], (m & (half - 1)) * (8 >> st));
             }
         }
 #pragma unroll
@@ -189,8 +211,11 @@ __device__ void fft_smem(C* buf, int L, int logL, const C* __restrict__ tw, int 
 // offsets from one base.
 constexpr int kFftThreads = 256;
 
-template <int CN, int LOGL>
+// (FP64 passes take R = 4 even where that leaves threads idle: a pass less is a set of twiddle
+// products less on the FP64 pipe, which half the threads keep busy)
+template <typename C, int CN, int LOGL>
 __host__ __device__ constexpr int fft_fixed_radix() {
+    if (sizeof(C) == 16) return LOGL < 4 ? LOGL : 4;
     int R = 4;
     while (R > 2 && ((1 << LOGL) >> R) * CN < kFftThreads) --R;
     return R < LOGL ? R : LOGL;
@@ -224,10 +249,7 @@ __device__ __forceinline__ void fft_pass_fixed(C* buf, const C* __restrict__ tw,
 #pragma unroll
             for (int m = 0; m < G; ++m) {
                 if (m & half) continue;
-                const C v = mul_root16(x[m + half], (m & (half - 1)) * (8 >> st));
-                const C u = x[m];
-                x[m] = cadd(u, v);
-                x[m + half] = csub(u, v);
+                butterfly16(x[m], x[m + half], (m & (half - 1)) * (8 >> st));
             }
         }
 #pragma unroll
@@ -239,7 +261,7 @@ __device__ __forceinline__ void fft_pass_fixed(C* buf, const C* __restrict__ tw,
 template <typename C, int CN, bool PAD, int LOGL, int S = 1>
 __device__ __forceinline__ void fft_smem_fixed(C* buf, const C* __restrict__ tw, int N) {
     if constexpr (S <= LOGL) {
-        constexpr int R = fft_fixed_radix<CN, LOGL>();
+        constexpr int R = fft_fixed_radix<C, CN, LOGL>();
         constexpr int lead = LOGL % R;
         constexpr int RR = (S == 1 && lead) ? lead : R;
         fft_pass_fixed<C, CN, PAD, LOGL, RR, S>(buf, tw, N);

@@ -83,6 +83,14 @@ template <> struct RecReader<float> {
     }
 };
 
+// Where the factor sqrt(K) dt_u = scale^2 of X' goes.  FP32: into the inputs, scale at a time, so
+// that nothing leaves the normal range.  FP64: into the split's factor 1/2, where it costs nothing
+// (two FP64 multiplications per real input otherwise).
+__device__ __forceinline__ float scaled_in(float v, float scale) { return (scale * v) * scale; }
+__device__ __forceinline__ double scaled_in(double v, double) { return v; }
+__device__ __forceinline__ float half_out(float) { return 0.5f; }
+__device__ __forceinline__ double half_out(double scale) { return 0.5 * (scale * scale); }
+
 struct SeqRows {   // the two real rows of complex sequence (pair, kind)
     int64_t ra, rb;   // record rows (m * 3 + c), -1 = zero row
     int64_t ma, mb;   // pixels receiving |A|^2 and |B|^2 (-1 = none)
@@ -107,13 +115,13 @@ __device__ __forceinline__ SeqRows seq_rows(int64_t pair, int kind, int64_t n_pi
 
 // Split Z_l / Z_{N-l} into the two real rows' spectra and accumulate the powers.
 template <typename T, typename C>
-__device__ __forceinline__ void emit(const SeqRows& sr, int64_t l, C zl, C zn, int64_t nl,
+__device__ __forceinline__ void emit(const SeqRows& sr, int64_t l, C zl, C zn, int64_t nl, T h,
                                      T* __restrict__ S, C* __restrict__ X, bool atomic) {
-    C A, B;
-    A.x = (T)0.5 * (zl.x + zn.x);
-    A.y = (T)0.5 * (zl.y - zn.y);
-    B.x = (T)0.5 * (zl.y + zn.y);
-    B.y = (T)0.5 * (zn.x - zl.x);
+    C A, B;   // h: half_out
+    A.x = h * (zl.x + zn.x);
+    A.y = h * (zl.y - zn.y);
+    B.x = h * (zl.y + zn.y);
+    B.y = h * (zn.x - zl.x);
     const T pa = A.x * A.x + A.y * A.y;
     const T pb = B.x * B.x + B.y * B.y;
     if (sr.ma >= 0) {
@@ -145,16 +153,16 @@ __global__ void spectrum_direct_kernel(RecReader<T> rd, int64_t n_pix, int N, in
         if (sr.ma < 0 && sr.mb < 0) continue;
         for (int j = threadIdx.x; j < N; j += blockDim.x) {
             C z;
-            z.x = sr.ra >= 0 ? (scale * rd(sr.ra, N, j)) * scale : (T)0;
-            z.y = sr.rb >= 0 ? (scale * rd(sr.rb, N, j)) * scale : (T)0;
+            z.x = sr.ra >= 0 ? scaled_in(rd(sr.ra, N, j), scale) : (T)0;
+            z.y = sr.rb >= 0 ? scaled_in(rd(sr.rb, N, j), scale) : (T)0;
             buf[fft_slot<1, true>(bitrev(j, logN), 0, sh)] = z;
         }
         __syncthreads();
         fft_smem<C, 1, true>(buf, N, logN, tw, N, sh);
         for (int l = threadIdx.x; l < nl; l += blockDim.x) {
             const int ln = (N - l) & (N - 1);
-            emit<T, C>(sr, l, buf[fft_slot<1, true>(l, 0, sh)], buf[fft_slot<1, true>(ln, 0, sh)], nl, S, X,
-                       false);
+            emit<T, C>(sr, l, buf[fft_slot<1, true>(l, 0, sh)], buf[fft_slot<1, true>(ln, 0, sh)], nl,
+                       half_out(scale), S, X, false);
         }
         __syncthreads();
     }
@@ -210,10 +218,7 @@ __device__ __forceinline__ void fft_regs(C* x) {
 #pragma unroll
         for (int m = 0; m < R; ++m) {
             if (m & half) continue;
-            const C v = mul_root16(x[m + half], (m & (half - 1)) * (8 / half));
-            const C u = x[m];
-            x[m] = cadd(u, v);
-            x[m + half] = csub(u, v);
+            butterfly16(x[m], x[m + half], (m & (half - 1)) * (8 / half));
         }
     }
 }
@@ -315,8 +320,8 @@ __global__ void __launch_bounds__(RegPlan<LOGN>::T, RegPlan<LOGN>::template min_
                 }
 #pragma unroll
                 for (int u = 0; u < kBatch; ++u) {
-                    v[i0 + u].x = (scale * rd.cvt_fp64(va[u])) * scale;
-                    v[i0 + u].y = (scale * rd.cvt(vb[u])) * scale;
+                    v[i0 + u].x = scaled_in(rd.cvt_fp64(va[u]), scale);
+                    v[i0 + u].y = scaled_in(rd.cvt(vb[u]), scale);
                 }
             }
         }
@@ -329,11 +334,12 @@ __global__ void __launch_bounds__(RegPlan<LOGN>::T, RegPlan<LOGN>::template min_
             // s = zl + zn, d = zl - zn: the two rows' spectra are A = (s.x, d.y) / 2 and
             // B = (s.y, -d.x) / 2
             const C sv = cadd(zl, zn), dv = csub(zl, zn);
+            const T h = half_out(scale);
             C A, B;
-            A.x = (T)0.5 * sv.x;
-            A.y = (T)0.5 * dv.y;
-            B.x = (T)0.5 * sv.y;
-            B.y = (T)-0.5 * dv.x;
+            A.x = h * sv.x;
+            A.y = h * dv.y;
+            B.x = h * sv.y;
+            B.y = -h * dv.x;
             const T pa = A.x * A.x + A.y * A.y, pb = B.x * B.x + B.y * B.y;
             if (X) {
                 X[(sr.ma * 3 + sr.ca) * nl + l] = A;
@@ -403,8 +409,8 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(T) == 4 ? 4 : 2)
             const int t = t0 + u * kFftThreads + threadIdx.x;
             if (t < N1 * CT) {
                 C z;
-                z.x = (scale * rd.cvt_fp64(va[u])) * scale;
-                z.y = (scale * rd.cvt(vb[u])) * scale;
+                z.x = scaled_in(rd.cvt_fp64(va[u]), scale);
+                z.y = scaled_in(rd.cvt(vb[u]), scale);
                 buf[bitrev(t / CT, logN1) * CT + t % CT] = z;
             }
         }
@@ -416,20 +422,24 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(T) == 4 ? 4 : 2)
     fft_smem_fixed<C, CT, false, LOGN1>(buf, tw, N);
     C* Ys = Y + seq * (int64_t)N;
     // twiddle exp(2 pi i j2 l1 / N), j2 = c0 + c, as tw[c0 l1] tw[c l1]: the second factor
-    // lies in the table's first CT * N1 entries, which stay in cache
+    // lies in the table's first CT * N1 entries, which stay in cache (FP64: from the table, whose
+    // scattered loads cost less than the product's four FP64 instructions)
     for (int t0 = 0; t0 < N1 * CT; t0 += kBatch * kFftThreads) {
         C w2[kBatch];
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) {
             const int t = t0 + u * kFftThreads + threadIdx.x;
-            w2[u] = t < N1 * CT ? tw[(t % CT) * (t / CT)] : C{};
+            w2[u] = t >= N1 * CT     ? C{}
+                    : sizeof(T) == 8 ? tw[((int64_t)(c0 + t % CT) * (t / CT)) & (N - 1)]
+                                     : tw[(t % CT) * (t / CT)];
         }
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) {
             const int t = t0 + u * kFftThreads + threadIdx.x;
             if (t < N1 * CT) {
                 const int c = t % CT, l1 = t / CT;
-                __stcs(Ys + (int64_t)l1 * N2 + c0 + c, cmul(buf[l1 * CT + c], cmul(wrow[l1], w2[u])));
+                const C w = sizeof(T) == 8 ? w2[u] : cmul(wrow[l1], w2[u]);
+                __stcs(Ys + (int64_t)l1 * N2 + c0 + c, cmul(buf[l1 * CT + c], w));
             }
         }
     }
@@ -441,7 +451,7 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(T) == 4 ? 4 : 2)
 // zeroing): every l <= N/2 has row l mod N1, which one CTA holds as l1 or as a mirror.
 template <typename T, int ROWS, int LOGN2>
 __global__ void __launch_bounds__(kFftThreads, sizeof(T) == 4 ? 4 : 2)
-    spectrum_pass2_kernel(int64_t n_pix, int N, int N1,
+    spectrum_pass2_kernel(int64_t n_pix, int N, int N1, T scale,
                           const typename V2<T>::type* __restrict__ tw,
                           const typename V2<T>::type* __restrict__ Y, T* __restrict__ S,
                           typename V2<T>::type* __restrict__ X, int64_t pair0) {
@@ -496,6 +506,7 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(T) == 4 ? 4 : 2)
     fft_smem_fixed<C, Cn, true, LOGN2>(buf, tw, N);
     const int64_t nl = N / 2 + 1;
     const int half = N / 2;
+    const T hs = half_out(scale), hs2 = hs * hs;
     // split: thread t takes row r = t % ROWS of side (t / ROWS) % 2 for every
     // (2 ROWS)-th l2; both are fixed per thread since kFftThreads is a multiple of 2 ROWS
     constexpr int L2STEP = kFftThreads / (2 * ROWS);
@@ -525,18 +536,18 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(T) == 4 ? 4 : 2)
             // and B = (s.y, -d.x) / 2
             const C sv = cadd(zl, zn), dv = csub(zl, zn);
             C A, B;
-            A.x = (T)0.5 * sv.x;
-            A.y = (T)0.5 * dv.y;
-            B.x = (T)0.5 * sv.y;
-            B.y = (T)-0.5 * dv.x;
+            A.x = hs * sv.x;
+            A.y = hs * dv.y;
+            B.x = hs * sv.y;
+            B.y = -hs * dv.x;
             T pa, pb;   // (x, y) of one pixel: pa = |A|^2 + |B|^2; (z0, z1): |A|^2, |B|^2
             if (kind < 2) {   // |A|^2 + |B|^2 = (|s|^2 + |d|^2) / 4
                 const C q = sumsq2(sv, dv);
-                pa = (T)0.25 * (q.x + q.y);
+                pa = hs2 * (q.x + q.y);
                 pb = (T)0;
             } else {
-                pa = (T)0.25 * (sv.x * sv.x + dv.y * dv.y);
-                pb = (T)0.25 * (sv.y * sv.y + dv.x * dv.x);
+                pa = hs2 * (sv.x * sv.x + dv.y * dv.y);
+                pb = hs2 * (sv.y * sv.y + dv.x * dv.x);
             }
             if (kind == 0) {          // (x0, y0)
                 pw0 += pa;
@@ -676,7 +687,7 @@ int run_spectrum(const void* record, int kind, int64_t n_pix, const lw_grid* g, 
         while (rows > 1 && sizeof(C) * (size_t)fft_slots(N2, logN2, 6 * rows) > 96 * 1024)
             rows >>= 1;
         const size_t smem = sizeof(C) * (size_t)fft_slots(N2, logN2, 6 * rows);
-        using K2 = void (*)(int64_t, int, int, const C*, const C*, T*, C*, int64_t);
+        using K2 = void (*)(int64_t, int, int, T, const C*, const C*, T*, C*, int64_t);
         const K2 k2s[3][4] = {
             {spectrum_pass2_kernel<T, 1, 6>, spectrum_pass2_kernel<T, 1, 7>,
              spectrum_pass2_kernel<T, 1, 8>, spectrum_pass2_kernel<T, 1, 9>},
@@ -693,7 +704,7 @@ int run_spectrum(const void* record, int kind, int64_t n_pix, const lw_grid* g, 
         for (int64_t p0 = 0; p0 < n_pairs; p0 += kPairsPerLaunch) {
             const int64_t np = std::min<int64_t>(kPairsPerLaunch, n_pairs - p0);
             dim3 grid((unsigned)groups, (unsigned)np);
-            kern<<<grid, kFftThreads, smem, st>>>(n_pix, (int)N, N1, tw, Y, S, X, p0);
+            kern<<<grid, kFftThreads, smem, st>>>(n_pix, (int)N, N1, scale, tw, Y, S, X, p0);
             if (launch_status() != LW_OK) return LW_ECUDA;
         }
         return LW_OK;
