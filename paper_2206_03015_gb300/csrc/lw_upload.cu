@@ -271,8 +271,7 @@ __global__ void order_range_kernel(const double* __restrict__ ends, int64_t n_e,
     }
 }
 
-__device__ __forceinline__ int order_bucket(const double* e, const unsigned long long* keys) {
-    const double lo = key_to_double(keys[0]), hi = key_to_double(keys[1]);
+__device__ __forceinline__ int order_bucket(const double* e, double lo, double hi) {
     const double v = first_tau(e);
     if (!(hi > lo) || !isfinite(v)) return 0;
     const double x = (v - lo) / (hi - lo) * kOrderBuckets;
@@ -284,11 +283,11 @@ __global__ void order_count_kernel(const double* __restrict__ ends, int64_t n_e,
                                    int32_t* __restrict__ counts) {
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n_e;
          k += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&counts[order_bucket(ends + 8 * k, keys)], 1);
+        atomicAdd(&counts[order_bucket(ends + 8 * k, key_to_double(keys[0]), key_to_double(keys[1]))], 1);
 }
 
 // Exclusive prefix sum of the bucket counts, in place (one CTA of 1024 threads).
-__global__ void __launch_bounds__(1024) order_scan_kernel(int32_t* counts) {
+__device__ void order_scan(int32_t* counts) {
     constexpr int kPer = kOrderBuckets / 1024;
     __shared__ int32_t s_sum[1024];
     int32_t v[kPer];
@@ -312,13 +311,88 @@ __global__ void __launch_bounds__(1024) order_scan_kernel(int32_t* counts) {
     }
 }
 
+__global__ void __launch_bounds__(1024) order_scan_kernel(int32_t* counts) { order_scan(counts); }
+
 __global__ void order_scatter_kernel(const double* __restrict__ ends, int64_t n_e,
                                      const unsigned long long* __restrict__ keys,
                                      int32_t* __restrict__ offsets, int32_t* __restrict__ order) {
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n_e;
          k += (int64_t)gridDim.x * blockDim.x) {
-        const int pos = atomicAdd(&offsets[order_bucket(ends + 8 * k, keys)], 1);
+        const int pos = atomicAdd(&offsets[order_bucket(ends + 8 * k, key_to_double(keys[0]), key_to_double(keys[1]))], 1);
         order[pos] = (int32_t)k;
+    }
+}
+
+// Ends, mean advance and order of up to kOrderOne electrons by one CTA, two per thread: the six
+// launches of the general form take 33 us of a stream, of which their work is a few.  Bound by the
+// one SM's FP64 pipe (16 electrons 10 us, 1,001 electrons 23 us), hence the limit.
+constexpr int kOrderOne = 2048;
+__global__ void __launch_bounds__(1024)
+    order_one_kernel(const double* __restrict__ t, int t_per_e, const double* __restrict__ r,
+                     int n_e, int64_t ns1, double* __restrict__ ends,
+                     double* __restrict__ span, int32_t* __restrict__ order) {
+    __shared__ int32_t s_counts[kOrderBuckets];
+    __shared__ double s_red[6][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int warps = min((n_e + 31) / 32, 32);   // with electrons
+    for (int b = threadIdx.x; b < kOrderBuckets; b += 1024) s_counts[b] = 0;
+    // v: smallest and negated largest tau, advance sums
+    double v[6] = {INFINITY, INFINITY, 0.0, 0.0, 0.0, 0.0}, tau[2] = {NAN, NAN};
+    for (int q = 0; q < 2; ++q) {
+        const int k = q * 1024 + (int)threadIdx.x;
+        if (k >= n_e) break;
+        const double* tk = t + (t_per_e ? k * ns1 : 0);
+        const double* x0 = r + 3 * (k * ns1);
+        const double* x1 = r + 3 * (k * ns1 + ns1 - 1);
+        const double e[8] = {tk[0], x0[0], x0[1], x0[2], tk[ns1 - 1], x1[0], x1[1], x1[2]};
+        for (int c = 0; c < 8; ++c) ends[8 * k + c] = e[c];
+        tau[q] = first_tau(e);
+        if (isfinite(tau[q])) {
+            v[0] = fmin(v[0], tau[q]);
+            v[1] = fmin(v[1], -tau[q]);
+            v[2] += first_tau(e + 4) - tau[q];
+            for (int c = 1; c < 4; ++c) v[2 + c] += e[4 + c] - e[c];
+        }
+    }
+    auto reduce = [&]() {
+        for (int o = 16; o > 0; o >>= 1)
+            for (int c = 0; c < 6; ++c) {
+                const double w = __shfl_xor_sync(0xffffffffu, v[c], o);
+                v[c] = c < 2 ? fmin(v[c], w) : v[c] + w;
+            }
+    };
+    if (warp < warps) {
+        reduce();
+        if (lane == 0)
+            for (int c = 0; c < 6; ++c) s_red[c][warp] = v[c];
+    }
+    __syncthreads();
+    if (warp == 0) {
+        for (int c = 0; c < 6; ++c) v[c] = lane < warps ? s_red[c][lane] : c < 2 ? INFINITY : 0.0;
+        reduce();
+        if (lane == 0) {
+            s_red[0][0] = v[0];
+            s_red[1][0] = (double)kOrderBuckets / (-v[1] - v[0]);   // buckets per tau
+            for (int c = 0; c < 4; ++c) span[c] = v[2 + c] / (double)n_e;
+        }
+    }
+    __syncthreads();
+    const double lo = s_red[0][0], per = s_red[1][0];
+    int bucket[2];
+    for (int q = 0; q < 2; ++q) {
+        if (q * 1024 + (int)threadIdx.x >= n_e) break;
+        // one tau, or none that is finite: bucket 0
+        const double x = (tau[q] - lo) * per;
+        bucket[q] = x > 0.0 ? (int)fmin(x, (double)(kOrderBuckets - 1)) : 0;
+        atomicAdd(&s_counts[bucket[q]], 1);
+    }
+    __syncthreads();
+    order_scan(s_counts);
+    __syncthreads();
+    for (int q = 0; q < 2; ++q) {
+        const int k = q * 1024 + (int)threadIdx.x;
+        if (k >= n_e) break;
+        order[atomicAdd(&s_counts[bucket[q]], 1)] = k;
     }
 }
 
@@ -434,9 +508,26 @@ extern "C" int lw_trajectories_upload(const lw_traj_in* in, int32_t sections, in
     }
     const int threads = 256;
     double* ends = reinterpret_cast<double*>(base + L.ends);
-    ends_kernel<<<grid_for(in->n_e, threads), threads, 0, st>>>(t, t_per_e, r, in->n_e, ns1,
-                                                                 ends);
+    int32_t* order = reinterpret_cast<int32_t*>(base + L.order);
+    OrderScratch* tmp = reinterpret_cast<OrderScratch*>(base + L.order_tmp);
+    const bool one = in->n_e <= kOrderOne;
+    if (one) {
+        order_one_kernel<<<1, 1024, 0, st>>>(t, t_per_e, r, (int)in->n_e, ns1, ends, tmp->span,
+                                             order);
+    } else {
+        const int ge = grid_for(in->n_e, threads);
+        ends_kernel<<<ge, threads, 0, st>>>(t, t_per_e, r, in->n_e, ns1, ends);
+        if (cudaMemsetAsync(tmp->counts, 0, sizeof(tmp->counts) + sizeof(tmp->span), st) !=
+            cudaSuccess)
+            return LW_ECUDA;
+        bounds_init_kernel<<<1, 1, 0, st>>>(tmp->keys);
+        order_range_kernel<<<ge, threads, 0, st>>>(ends, in->n_e, tmp->keys, tmp->span);
+        order_count_kernel<<<ge, threads, 0, st>>>(ends, in->n_e, tmp->keys, tmp->counts);
+        order_scan_kernel<<<1, 1024, 0, st>>>(tmp->counts);
+        order_scatter_kernel<<<ge, threads, 0, st>>>(ends, in->n_e, tmp->keys, tmp->counts, order);
+    }
     if (launch_status() != LW_OK) return LW_ECUDA;
+    v.order = order;
     v.ends = ends;
     float4* scan = nullptr;
     float* field = nullptr;
@@ -461,22 +552,6 @@ extern "C" int lw_trajectories_upload(const lw_traj_in* in, int32_t sections, in
                                           anchor,
                                           (sections & LW_SECTION_FP64) ? 1 : 0, status);
     if (launch_status() != LW_OK) return LW_ECUDA;
-    {
-        int32_t* order = reinterpret_cast<int32_t*>(base + L.order);
-        OrderScratch* tmp = reinterpret_cast<OrderScratch*>(base + L.order_tmp);
-        unsigned long long* keys = tmp->keys;
-        int32_t* counts = tmp->counts;
-        if (cudaMemsetAsync(counts, 0, sizeof(tmp->counts) + sizeof(tmp->span), st) != cudaSuccess)
-            return LW_ECUDA;
-        bounds_init_kernel<<<1, 1, 0, st>>>(keys);
-        const int ge = grid_for(in->n_e, threads);
-        order_range_kernel<<<ge, threads, 0, st>>>(ends, in->n_e, keys, tmp->span);
-        order_count_kernel<<<ge, threads, 0, st>>>(ends, in->n_e, keys, counts);
-        order_scan_kernel<<<1, 1024, 0, st>>>(counts);
-        order_scatter_kernel<<<ge, threads, 0, st>>>(ends, in->n_e, keys, counts, order);
-        if (launch_status() != LW_OK) return LW_ECUDA;
-        v.order = order;
-    }
     *out = v;
     *ws_bytes = L.total;
     return LW_OK;
