@@ -1701,8 +1701,8 @@ extern "C" int lw_deposit_time_domain(const lw_traj* traj, const lw_detector* de
     const size_t smem = kMixStages * stage_bytes(traj->block);   // staging ring
     // dense tiles (decided on the device, walk_tile) are walked by a launch of their own where the
     // grid can hold that many points per step
-    if ((double)grid->n_bins > kWalkDensity * (double)traj->n_s) {
-        a.span = traj_span(traj);
+    if ((double)grid->n_bins > kWalkDensity * (double)traj->n_s) a.span = traj_span(traj);
+    if (a.span) {
         DepositArgs w = a;
         const int64_t wx = (det->n_pix + kMixThreads - 1) / kMixThreads;
         const int64_t rows = std::max<int64_t>(1, 2 * two_waves / wx);

@@ -42,11 +42,9 @@ struct OrderScratch {
     int32_t counts[kOrderBuckets];
     double span[4];
 };
-inline const double* traj_span(const lw_traj* t) {
-    const char* order = reinterpret_cast<const char*>(t->order);
-    return reinterpret_cast<const OrderScratch*>(order + align256(sizeof(int32_t) * (size_t)t->n_e))
-        ->span;
-}
+// The mean advance of a view, or null where the view's pointers do not lie as the upload lays them
+// out (an order of the caller's own, or none; fewer electrons): there is none to read then.
+const double* traj_span(const lw_traj* t);
 
 __device__ __forceinline__ void status_or(int32_t* st, int bits) {
     if (st && bits) atomicOr(st, bits);

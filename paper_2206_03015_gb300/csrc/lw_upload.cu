@@ -445,6 +445,19 @@ int grid_for(int64_t work, int threads) {
 }
 
 }  // namespace
+
+const double* traj_span(const lw_traj* t) {
+    if (t->n_e < 1 || t->n_s < 1 || t->block < 1) return nullptr;
+    const TrajLayout L = make_layout(t->n_e, t->n_s, t->t_per_electron, t->sections, t->block);
+    // compared as integers: the pointers of such a view may belong to different allocations
+    const uintptr_t base = reinterpret_cast<uintptr_t>(t->input_status);
+    if (reinterpret_cast<uintptr_t>(t->ends) != base + L.ends ||
+        reinterpret_cast<uintptr_t>(t->anchor) != base + L.anchor ||
+        reinterpret_cast<uintptr_t>(t->order) != base + L.order)
+        return nullptr;
+    return reinterpret_cast<const OrderScratch*>(base + L.order_tmp)->span;
+}
+
 }  // namespace lw
 
 using namespace lw;

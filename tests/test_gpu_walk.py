@@ -10,7 +10,7 @@ import pytest
 torch = pytest.importorskip("torch")
 
 import oracle  # noqa: E402
-from gpu_cases import gpu_bounds, gpu_run, oracle_run  # noqa: E402
+from gpu_cases import gpu_bounds, gpu_run, oracle_run, record_value  # noqa: E402
 from paper_2206_03015_gb300 import lw  # noqa: E402
 from workloads import simple  # noqa: E402
 
@@ -86,3 +86,19 @@ def test_tiles_on_both_sides_of_the_threshold():
     want = oracle_run(tr, n_hat, grid, spectrum=False)
     assert np.abs(got["rec"] - want["rec"]).max() <= 1e-4 * np.abs(want["rec"]).max()
     assert got["status"] == want["status"]
+
+
+def test_view_with_another_order():
+    """A view whose order was taken out, or stands elsewhere, has no mean advance to decide by: its
+    dense tiles are searched and its record is the same."""
+    tr = simple.transverse_oscillation(3, 400, 1e-17, 0.999, 0.01, 97.0, seed=4)
+    n_hat = np.array([[0.0, 0.0, 1.0], [0.01, 0.0, np.sqrt(1 - 1e-4)]])
+    grid = _whole(900)(*gpu_bounds(tr, n_hat))
+    want = oracle_run(tr, n_hat, grid, spectrum=False)["rec"]
+    traj = lw.lw_trajectories_upload(tr.t, tr.r, tr.beta, tr.beta_dot)
+    own = traj.order().clone()
+    det = lw.Detector(n_hat)
+    for order in (traj.view.order, None, own.data_ptr()):
+        traj.view.order = order
+        got = record_value(lw.lw_deposit_time_domain(traj, det, grid, lw.LW_MIXED), lw.LW_MIXED)
+        assert np.abs(got - want).max() <= 1e-4 * np.abs(want).max()
