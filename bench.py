@@ -538,11 +538,16 @@ def run_ours(args, rank, world, dist):
     result["accuracy"] = acc
     result["status"] = {"mixed": st_m, "note": "8 = last arrival on grid point n_bins (clipped)"}
 
-    # launches of our kernels per timed step: upload (ends, prepare, and the electron
-    # order: key init, range, count, scan, scatter), deposit (1), spectrum (twiddle, then
-    # pass 1 + pass 2, or the direct kernel up to 4096 bins)
-    spec_k = 2 if grid.n_bins <= 4096 else 3
-    result["gpu_launches"] = args.steps * (7 + 1 + spec_k)
+    # launches of our kernels per timed step: upload (prepare, and ends and electron order in
+    # one launch up to 2,048 electrons, else ends, key init, range, count, scan, scatter),
+    # deposit (search, precision check, and the walk of dense tiles where the grid can hold
+    # as many points per step as the record's line says), spectrum (twiddle and one transform
+    # kernel, or the two passes above 16,384 bins and above 4,096 with fewer than 76 pixel pairs)
+    upload_k = 2 if tr.n_e <= 2048 else 7
+    line = {lw.LW_MIXED_F32X4: 1.0, lw.LW_MIXED_F32: 1.4}.get(MIX, 1.8)
+    deposit_k = 3 if grid.n_bins > line * tr.n_s else 2
+    spec_k = 2 if grid.n_bins <= 4096 or (grid.n_bins <= 16384 and det.n_pix > 150) else 3
+    result["gpu_launches"] = args.steps * (upload_k + deposit_k + spec_k)
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         result["cpu_baseline"] = cpu_baseline(w, grid, S_m, args)
     return result

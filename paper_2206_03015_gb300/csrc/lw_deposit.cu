@@ -607,11 +607,19 @@ __device__ __forceinline__ int frac_floor(float f) { return f >= 1.0f ? 1 : (f <
 // so that the record updates of a warp are consecutive grid points of one pixel.  A grid point
 // belongs to the same step as in the search (the first sample whose coordinate reaches it; the
 // run's bounds ja .. ja + K - 1 go to the first and the last step).
-// The samples of a segment cost about 90 instructions per pixel whatever their grid points, and a
-// round of 32 grid points about 18, against 32 x 7.2 by search: the walk is the cheaper one above
-// kWalkDensity grid points per step.  2,048 co-located electrons x 4,096 steps x 1,024 pixels x
-// 16,384 bins (1 to 5 grid points per step): 238 ms by search, 82 ms walked.
-constexpr double kWalkDensity = 0.45;
+// The samples cost about the same whatever their grid points, a grid point about a ninth of what
+// its search does.  512 co-located electrons x 4,096 steps x 1,024 pixels, search and walk at
+// 0.7, 1.0, 1.5 and 3 grid points per step: interleaved FP32 record 13.2 and 14.4, 15.8 and 14.5,
+// 24.6 and 17.5, 48 and 21 ms; FP32 rows (1.2, 1.5, 2) 21.7 and 24.4, 25.5 and 24.3, 33 and 21; FP64
+// record 14.9 and 20.2, 18.5 and 20.8, 28.6 and 35, (2, 3) 37 and 28, 56 and 47; compensated record
+// 20 and 26, 26 and 28, 40 and 54, (2, 3, 6) 52 and 48, 80 and 86, 164 and 147.  The line lies where
+// the walk gains on electrons that start together; those of a bunch gain earlier (1,000 electrons, 1.0
+// per step, 256 pixels: 42 and 25 ms).  2,048 co-located electrons x 4,096 steps x 1,024 pixels x 16,384
+// bins (1 to 5 grid points per step): 238 ms by search, 82 ms walked.
+template <int ACC>
+__host__ __device__ constexpr double walk_density() {
+    return ACC == kAccF32X4 ? 1.0 : ACC == kAccF32 ? 1.4 : ACC == kAccKahan ? 4.0 : 1.8;
+}
 constexpr int kWalkTile = 512;  // pixels that share a decision
 constexpr int kWalkMap = 256;   // grid points of a segment mapped to steps at a time
 
@@ -699,10 +707,10 @@ __device__ __forceinline__ void walk_block(const float4* s_scan, const float4* s
 // only.  A test of every electron, by each of the search's CTAs, cost more than it sorted out
 // (36 FP64 instructions: 10 % of a 1,001-electron step).
 __device__ __noinline__ bool walk_tile(const double* span, const double* n_hat, int64_t n_pix,
-                                       int64_t pix, double steps, double inv_dtu) {
+                                       int64_t pix, double points, double inv_dtu) {
     const double* n = n_hat + 3 * min(pix, n_pix - 1);
     const double nr = (n[0] * span[1] + n[1] * span[2]) - (1.0 - n[2]) * span[3];
-    return (span[0] - nr * kInvC0) * inv_dtu > kWalkDensity * steps;
+    return (span[0] - nr * kInvC0) * inv_dtu > points;
 }
 
 // The work of one CTA: pixel tile `tile` (kMixThreads * PIX pixels) and electron
@@ -1426,11 +1434,12 @@ __global__ void __launch_bounds__(kFp64Threads) deposit_fp64_kernel(DepositArgs 
 }
 
 // walk_tile for the CTA (thread 0 decides)
+template <int ACC>
 __device__ __forceinline__ bool tile_is_dense(const DepositArgs& p, int64_t pix0) {
     int dense = 0;
     if (threadIdx.x == 0)
         dense = walk_tile(p.span, p.n_hat, p.n_pix, pix0 / kWalkTile * kWalkTile + kWalkTile / 2,
-                          (double)(p.ns1 - 1), p.inv_dtu);
+                          walk_density<ACC>() * (double)(p.ns1 - 1), p.inv_dtu);
     return __syncthreads_or(dense) != 0;
 }
 
@@ -1439,7 +1448,7 @@ __global__ void __launch_bounds__(kMixThreads, kMixMinBlocks) deposit_mixed_kern
     // the precision check launched after this grid (programmatic dependent launch) may
     // start once every CTA of this grid has started: it fills the SMs of the last wave
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (p.span && tile_is_dense(p, (int64_t)blockIdx.x * (kMixThreads * PIX))) return;
+    if (p.span && tile_is_dense<ACC>(p, (int64_t)blockIdx.x * (kMixThreads * PIX))) return;
     const int bits =
         mixed_cta<PIX, ACC, FL, kSearch, SPLIT>(p, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.z);
     block_status_or(p.status, bits);
@@ -1449,7 +1458,7 @@ __global__ void __launch_bounds__(kMixThreads, kMixMinBlocks) deposit_mixed_kern
 // tiles is about four waves of CTAs that end at once, 5 us).
 template <int ACC, int FL>
 __global__ void __launch_bounds__(kMixThreads, kMixMinBlocks) deposit_walk_kernel(DepositArgs p) {
-    if (!tile_is_dense(p, (int64_t)blockIdx.x * kMixThreads)) return;
+    if (!tile_is_dense<ACC>(p, (int64_t)blockIdx.x * kMixThreads)) return;
     const int bits = mixed_cta<1, ACC, FL, kWalk, true>(p, blockIdx.x, blockIdx.y, blockIdx.z,
                                                         gridDim.z);
     block_status_or(p.status, bits);
@@ -1701,7 +1710,11 @@ extern "C" int lw_deposit_time_domain(const lw_traj* traj, const lw_detector* de
     const size_t smem = kMixStages * stage_bytes(traj->block);   // staging ring
     // dense tiles (decided on the device, walk_tile) are walked by a launch of their own where the
     // grid can hold that many points per step
-    if ((double)grid->n_bins > kWalkDensity * (double)traj->n_s) a.span = traj_span(traj);
+    const double density = acc_of(precision) == kAccF32X4 ? walk_density<kAccF32X4>()
+                           : acc_of(precision) == kAccF32   ? walk_density<kAccF32>()
+                           : acc_of(precision) == kAccKahan ? walk_density<kAccKahan>()
+                                                            : walk_density<kAccF64>();
+    if ((double)grid->n_bins > density * (double)traj->n_s) a.span = traj_span(traj);
     if (a.span) {
         DepositArgs w = a;
         const int64_t wx = (det->n_pix + kMixThreads - 1) / kMixThreads;

@@ -1,4 +1,4 @@
-"""Mixed deposit of dense grids (more than about half a grid point per step), whose blocks are walked
+"""Mixed deposit of dense grids (from about one grid point per step on), whose blocks are walked
 sample by sample, at the edges of the walk: densities on both sides of its threshold, segments of
 32 samples with remainders, more grid points per segment than its map holds (256), one block and
 several, electrons of very different densities in one launch, pixel tiles on both sides of the
@@ -35,7 +35,7 @@ def _whole(n_bins):
 
 
 @pytest.mark.parametrize("n_s", [1, 31, 32, 33, 511, 512, 513, 1100])
-@pytest.mark.parametrize("per_step", [0.4, 0.5, 3.3, 12.0])
+@pytest.mark.parametrize("per_step", [0.4, 0.5, 0.95, 1.05, 3.3, 12.0])
 def test_steps_and_density(n_s, per_step):
     tr = simple.transverse_oscillation(2, n_s, 1e-17, 0.999, 0.01, 97.0, seed=n_s)
     _compare(tr, 3, _whole(max(4, int(n_s * per_step))), lw.LW_MIXED_F32X4)
@@ -86,6 +86,13 @@ def test_tiles_on_both_sides_of_the_threshold():
     want = oracle_run(tr, n_hat, grid, spectrum=False)
     assert np.abs(got["rec"] - want["rec"]).max() <= 1e-4 * np.abs(want["rec"]).max()
     assert got["status"] == want["status"]
+
+
+@pytest.mark.parametrize("prec", [lw.LW_MIXED, lw.LW_MIXED_KAHAN, lw.LW_MIXED_F32])
+@pytest.mark.parametrize("per_step", [1.35, 1.45, 1.75, 1.85, 3.9, 4.2, 7.0])
+def test_density_of_each_record(prec, per_step):
+    tr = simple.transverse_oscillation(2, 300, 1e-17, 0.999, 0.01, 97.0, seed=9)
+    _compare(tr, 3, _whole(int(300 * per_step * 1.02)), prec)
 
 
 def test_view_with_another_order():
