@@ -607,15 +607,19 @@ __device__ __forceinline__ int frac_floor(float f) { return f >= 1.0f ? 1 : (f <
 // so that the record updates of a warp are consecutive grid points of one pixel.  A grid point
 // belongs to the same step as in the search (the first sample whose coordinate reaches it; the
 // run's bounds ja .. ja + K - 1 go to the first and the last step).
-// The samples cost about the same whatever their grid points, a grid point about a ninth of what
-// its search does.  512 co-located electrons x 4,096 steps x 1,024 pixels, search and walk at
-// 0.7, 1.0, 1.5 and 3 grid points per step: interleaved FP32 record 13.2 and 14.4, 15.8 and 14.5,
-// 24.6 and 17.5, 48 and 21 ms; FP32 rows (1.2, 1.5, 2) 21.7 and 24.4, 25.5 and 24.3, 33 and 21; FP64
-// record 14.9 and 20.2, 18.5 and 20.8, 28.6 and 35, (2, 3) 37 and 28, 56 and 47; compensated record
-// 20 and 26, 26 and 28, 40 and 54, (2, 3, 6) 52 and 48, 80 and 86, 164 and 147.  The line lies where
-// the walk gains on electrons that start together; those of a bunch gain earlier (1,000 electrons, 1.0
-// per step, 256 pixels: 42 and 25 ms).  2,048 co-located electrons x 4,096 steps x 1,024 pixels x 16,384
-// bins (1 to 5 grid points per step): 238 ms by search, 82 ms walked.
+// A contribution is the search's to the bit: the samples keep their end terms and scale apart (five
+// words), and a grid point weights and sums them in the search's operations.  Interpolating between
+// fields already multiplied out (four words, 6 % faster: 17.4 and 18.6 ms below) rounds otherwise and
+// moved a gradient over 2,048 electrons, which adds up what they share.
+// 512 co-located electrons x 4,096 steps x 1,024 pixels, search and walk at 1.05, 1.5 and 3 grid
+// points per step: interleaved FP32 record 18.9 and 18.6, 24.6 and 18.8, 48 and 23 ms; FP32 rows
+// (1.45, 2) 27.0 and 26.0, 33 and 23; FP64 record (1.85, 2, 3) 38 and 35, 37 and 28, 56 and 47;
+// compensated record (4.1, 6, 10) 118 and 101, 164 and 131, 288 and 223.  The line lies where
+// the walk gains on electrons that start together; those of a bunch gain earlier (1,000 electrons x
+// 10,000 steps x 256 pixels: interleaved record at 1.05 44 and 27, FP32 rows at 1.45 63 and 38, FP64
+// record at 1.85 92 and 65 ms; the compensated record loses there, at 4.1 356 and 386).
+// 2,048 co-located electrons x 4,096 steps x 1,024 pixels x 16,384 bins (1 to 5 grid points per
+// step): 238 ms by search, 83 ms walked.
 template <int ACC>
 __host__ __device__ constexpr double walk_density() {
     return ACC == kAccF32X4 ? 1.0 : ACC == kAccF32 ? 1.4 : ACC == kAccKahan ? 4.0 : 1.8;
@@ -623,18 +627,24 @@ __host__ __device__ constexpr double walk_density() {
 constexpr int kWalkTile = 512;  // pixels that share a decision
 constexpr int kWalkMap = 256;   // grid points of a segment mapped to steps at a time
 
+// One warp's walk (in its job table's place).  Entry 0: the sample before the segment of 32, entry
+// 1 + l: the segment's sample l, each with its coordinate, its end terms and their scale.
+struct WalkStage {
+    float4 xt[33];
+    float sc[33];
+    unsigned char map[kWalkMap];   // grid point of the segment -> sample at the step's end
+};
+static_assert(sizeof(WalkStage) <= sizeof(int2) * kJobTable, "a warp's walk lies in its job table");
+
 template <int PIX, int ACC, int FL>
 __device__ __forceinline__ void walk_block(const float4* s_scan, const float4* s_f4,
                                         const float2* s_f2, int ns, const float4* s_wh,
                                         const int4* s_job, int2 K2, int2 JA2, float s32,
                                         float inv_sc, float c0_over_R, int64_t n_bins,
-                                        unsigned char* tile_rec, float4* stage,
-                                        unsigned char* map) {
+                                        unsigned char* tile_rec, WalkStage& st) {
     const int lane = threadIdx.x & 31;
     const uint64_t row_bytes =
         4ull * (ACC == kAccF32X4 ? 4 : ACC == kAccF32 ? 3 : 6) * (uint64_t)n_bins;
-    // stage[0]: the sample before the segment, stage[1 + l]: the segment's sample l, each
-    // (coordinate, field)
     for (int slot = 0; slot < 32 * PIX; ++slot) {   // s_wh, s_job: the warp's slots
         const int K = __shfl_sync(0xffffffffu, slot % PIX ? K2.y : K2.x, slot / PIX);
         if (K == 0) continue;
@@ -674,24 +684,30 @@ __device__ __forceinline__ void walk_block(const float4* s_scan, const float4* s
                 if (lane == 0) before = Jc;
             }
             __syncwarp();   // the segment before is read
-            if (r0 > 0 && lane == 0) stage[0] = stage[32];
+            if (r0 > 0 && lane == 0) {
+                st.xt[0] = st.xt[32];
+                st.sc[0] = st.sc[32];
+            }
             __syncwarp();
-            stage[1 + lane] = make_float4(x, txy.x * sc, txy.y * sc, tz * sc);
+            st.xt[1 + lane] = make_float4(x, txy.x, txy.y, tz);
+            st.sc[1 + lane] = sc;
             const int Je = __shfl_sync(0xffffffffu, J, 31);
             for (int b0 = Jc; b0 < Je; b0 += kWalkMap) {   // grid points b0 + 1 .. b0 + kWalkMap
                 const int z = min(J - b0, kWalkMap);
-                for (int t = max(before - b0, 0); t < z; ++t) map[t] = (unsigned char)lane;
+                for (int t = max(before - b0, 0); t < z; ++t) st.map[t] = (unsigned char)lane;
                 __syncwarp();
                 const int n = min(Je - b0, kWalkMap);
                 for (int t = lane; t < n; t += 32) {
-                    const int e = map[t];   // step from sample e - 1 to sample e of the segment
-                    const float4 a = stage[e], b = stage[e + 1];
+                    const int e = st.map[t];   // step from sample e - 1 to sample e of the segment
+                    const float4 a = st.xt[e], b = st.xt[e + 1];
                     const int j = b0 + 1 + t;
                     const float tJ = __fsub_rn((float)j, f);
                     const float du = __fsub_rn(b.x, a.x);
                     const float wb = du > 0.0f ? __fdividef(__fsub_rn(tJ, a.x), du) : 0.0f;
-                    deposit3_row<ACC>(row, j + jb.x, n_bins, fmaf(wb, b.y - a.y, a.y),
-                                      fmaf(wb, b.z - a.z, a.z), fmaf(wb, b.w - a.w, a.w));
+                    // the search's operations, so that a contribution is the same to the bit
+                    const float sa = (1.0f - wb) * st.sc[e], sb = wb * st.sc[e + 1];
+                    deposit3_row<ACC>(row, j + jb.x, n_bins, fmaf(a.y, sa, b.y * sb),
+                                      fmaf(a.z, sa, b.z * sb), fmaf(a.w, sa, b.w * sb));
                 }
                 __syncwarp();   // the map is rewritten
             }
@@ -1032,8 +1048,8 @@ __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int
                 walk_block<PIX, ACC, FL>(
                     s_scan, s_f4, s_f2, ns, s_wh + wslot, s_job + wslot,
                     make_int2(K[0], K[PIX - 1]), make_int2(JA[0], JA[PIX - 1]), s32, inv_sc,
-                    c0_over_R, p.n_bins, tile_rec, reinterpret_cast<float4*>(&s_tab[warp][0]),
-                    reinterpret_cast<unsigned char*>(&s_tab[warp][kJobTable / 2 + 4]));
+                    c0_over_R, p.n_bins, tile_rec,
+                    *reinterpret_cast<WalkStage*>(&s_tab[warp][0]));
                 continue;
             }
             // Grid point j (absolute) of slot sl with block data I, f, xe (coordinate of the
@@ -1716,19 +1732,18 @@ extern "C" int lw_deposit_time_domain(const lw_traj* traj, const lw_detector* de
                                                             : walk_density<kAccF64>();
     if ((double)grid->n_bins > density * (double)traj->n_s) a.span = traj_span(traj);
     if (a.span) {
-        DepositArgs w = a;
+        // electrons in the search's chunks and order: an FP32 record is rounded at every addition,
+        // and chunks of four electrons instead of one moved dL/dw0 of 2,048 electrons by 0.9 to 1.5
+        // of its run-to-run deviations (now 0.2 to 0.6)
         const int64_t wx = (det->n_pix + kMixThreads - 1) / kMixThreads;
-        const int64_t rows = std::max<int64_t>(1, 2 * two_waves / wx);
-        w.e_chunk = (int)std::max<int64_t>(std::max<int64_t>(traj->n_e / rows, 1),
-                                           (traj->n_e + 65534) / 65535);
-        const int64_t chunks = (traj->n_e + w.e_chunk - 1) / w.e_chunk;
+        const int64_t chunks = (traj->n_e + a.e_chunk - 1) / a.e_chunk;
         const int64_t parts = std::min<int64_t>(std::min<int64_t>(nbs, 64),
                                                 (two_waves + wx * chunks - 1) / (wx * chunks));
         const MixedKernel wk = walk_kernel(acc_of(precision), field_flags);
         if (cudaFuncSetAttribute(wk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
             cudaSuccess)
             return LW_ECUDA;
-        wk<<<dim3((unsigned)wx, (unsigned)chunks, (unsigned)parts), kMixThreads, smem, st>>>(w);
+        wk<<<dim3((unsigned)wx, (unsigned)chunks, (unsigned)parts), kMixThreads, smem, st>>>(a);
         if (launch_status() != LW_OK) return LW_ECUDA;
     }
     // static tables + double-buffered staging exceed the 48 KB default: opt in
