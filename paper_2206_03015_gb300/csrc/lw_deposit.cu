@@ -613,16 +613,18 @@ __device__ __forceinline__ int frac_floor(float f) { return f >= 1.0f ? 1 : (f <
 // moved a gradient over 2,048 electrons, which adds up what they share.
 // 512 co-located electrons x 4,096 steps x 1,024 pixels, search and walk at 1.05, 1.5 and 3 grid
 // points per step: interleaved FP32 record 18.9 and 18.6, 24.6 and 18.8, 48 and 23 ms; FP32 rows
-// (1.45, 2) 27.0 and 26.0, 33 and 23; FP64 record (1.85, 2, 3) 38 and 35, 37 and 28, 56 and 47;
-// compensated record (4.1, 6, 10) 118 and 101, 164 and 131, 288 and 223.  The line lies where
-// the walk gains on electrons that start together; those of a bunch gain earlier (1,000 electrons x
-// 10,000 steps x 256 pixels: interleaved record at 1.05 44 and 27, FP32 rows at 1.45 63 and 38, FP64
-// record at 1.85 92 and 65 ms; the compensated record loses there, at 4.1 356 and 386).
+// (1.45, 2) 27.0 and 26.0, 33 and 23; FP64 record (1.85, 2, 3) 38 and 35, 37 and 28, 56 and 47.
+// The line lies where the walk gains on electrons that start together; those of a bunch gain earlier
+// (1,000 electrons x 10,000 steps x 256 pixels: interleaved record at 1.05 44 and 27, FP32 rows at
+// 1.45 63 and 38, FP64 record at 1.85 92 and 65 ms).  The compensated record is always searched: its
+// returning additions of neighbouring grid points, which the walk puts side by side, wait for one
+// another (4.1, 6 and 10 points per step: the 512 electrons 118 and 101, 164 and 131, 288 and 223 ms,
+// but the bunch 356 and 386, 522 and 551; 400 electrons of it 75 and 87, 105 and 117, 175 and 193).
 // 2,048 co-located electrons x 4,096 steps x 1,024 pixels x 16,384 bins (1 to 5 grid points per
 // step): 238 ms by search, 83 ms walked.
 template <int ACC>
 __host__ __device__ constexpr double walk_density() {
-    return ACC == kAccF32X4 ? 1.0 : ACC == kAccF32 ? 1.4 : ACC == kAccKahan ? 4.0 : 1.8;
+    return ACC == kAccF32X4 ? 1.0 : ACC == kAccF32 ? 1.4 : 1.8;
 }
 constexpr int kWalkTile = 512;  // pixels that share a decision
 constexpr int kWalkMap = 256;   // grid points of a segment mapped to steps at a time
@@ -1464,7 +1466,8 @@ __global__ void __launch_bounds__(kMixThreads, kMixMinBlocks) deposit_mixed_kern
     // the precision check launched after this grid (programmatic dependent launch) may
     // start once every CTA of this grid has started: it fills the SMs of the last wave
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (p.span && tile_is_dense<ACC>(p, (int64_t)blockIdx.x * (kMixThreads * PIX))) return;
+    if (ACC != kAccKahan && p.span && tile_is_dense<ACC>(p, (int64_t)blockIdx.x * (kMixThreads * PIX)))
+        return;
     const int bits =
         mixed_cta<PIX, ACC, FL, kSearch, SPLIT>(p, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.z);
     block_status_or(p.status, bits);
@@ -1588,8 +1591,7 @@ MixedKernel walk_kernel_fl(uint32_t fl) {
            : fl == 2 ? deposit_walk_kernel<ACC, 2> : deposit_walk_kernel<ACC, 3>;
 }
 MixedKernel walk_kernel(int acc, uint32_t fl) {
-    return acc == kAccKahan ? walk_kernel_fl<kAccKahan>(fl)
-           : acc == kAccF32 ? walk_kernel_fl<kAccF32>(fl)
+    return acc == kAccF32 ? walk_kernel_fl<kAccF32>(fl)
            : acc == kAccF32X4 ? walk_kernel_fl<kAccF32X4>(fl) : walk_kernel_fl<kAccF64>(fl);
 }
 using CheckKernel = void (*)(DepositArgs, int);
@@ -1726,11 +1728,11 @@ extern "C" int lw_deposit_time_domain(const lw_traj* traj, const lw_detector* de
     const size_t smem = kMixStages * stage_bytes(traj->block);   // staging ring
     // dense tiles (decided on the device, walk_tile) are walked by a launch of their own where the
     // grid can hold that many points per step
-    const double density = acc_of(precision) == kAccF32X4 ? walk_density<kAccF32X4>()
-                           : acc_of(precision) == kAccF32   ? walk_density<kAccF32>()
-                           : acc_of(precision) == kAccKahan ? walk_density<kAccKahan>()
-                                                            : walk_density<kAccF64>();
-    if ((double)grid->n_bins > density * (double)traj->n_s) a.span = traj_span(traj);
+    const int acc = acc_of(precision);
+    const double density = acc == kAccF32X4 ? walk_density<kAccF32X4>()
+                           : acc == kAccF32 ? walk_density<kAccF32>() : walk_density<kAccF64>();
+    if (acc != kAccKahan && (double)grid->n_bins > density * (double)traj->n_s)
+        a.span = traj_span(traj);
     if (a.span) {
         // electrons in the search's chunks and order: an FP32 record is rounded at every addition,
         // and chunks of four electrons instead of one moved dL/dw0 of 2,048 electrons by 0.9 to 1.5
@@ -1739,7 +1741,7 @@ extern "C" int lw_deposit_time_domain(const lw_traj* traj, const lw_detector* de
         const int64_t chunks = (traj->n_e + a.e_chunk - 1) / a.e_chunk;
         const int64_t parts = std::min<int64_t>(std::min<int64_t>(nbs, 64),
                                                 (two_waves + wx * chunks - 1) / (wx * chunks));
-        const MixedKernel wk = walk_kernel(acc_of(precision), field_flags);
+        const MixedKernel wk = walk_kernel(acc, field_flags);
         if (cudaFuncSetAttribute(wk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
             cudaSuccess)
             return LW_ECUDA;

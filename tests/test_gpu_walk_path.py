@@ -7,7 +7,7 @@ import pytest
 torch = pytest.importorskip("torch")
 
 from paper_2206_03015_gb300 import lw  # noqa: E402
-from workloads import simple  # noqa: E402
+from workloads import configs, simple  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -24,11 +24,13 @@ def _grid(traj, det, n_bins):
 
 
 def _searched(traj):
-    """The same trajectories as a view without the upload's order, whose tiles are all searched."""
+    """The same trajectories as a view whose order (the same one) stands elsewhere, so that it has no
+    mean advance: its tiles are all searched."""
     view = lw.lw_traj.from_buffer_copy(traj.view)
-    view.order = None
+    order = traj.order().clone()
+    view.order = order.data_ptr()
     out = lw.Trajectories(traj.ws, view)
-    out._inputs = getattr(traj, "_inputs", None)
+    out._keep = order, getattr(traj, "_inputs", None)
     return out
 
 
@@ -56,49 +58,71 @@ def test_walk_and_search_agree_to_the_bit(prec, flags, n_s, per_step, block):
 def _span(traj):
     """The mean advance that the upload stores behind the order: after two keys and 4,096 counters."""
     at = traj.view.order + (4 * traj.n_e + 255) // 256 * 256 + 16 + 4 * 4096 - traj.ws.data_ptr()
-    return traj.ws[at:at + 32].view(torch.float64).cpu().numpy()
+    return traj.ws[at:at + 32].view(torch.float64)
 
 
-def _dense(traj, n_hat, grid, line):
-    """Per tile of 512 pixels: whether its middle pixel's mean advance is above the line."""
-    span = _span(traj)
-    mid = n_hat[np.minimum(np.arange(0, len(n_hat), 512) + 256, len(n_hat) - 1)]
-    adv = span[0] - (mid[:, 0] * span[1] + mid[:, 1] * span[2]
-                     - (1.0 - mid[:, 2]) * span[3]) / 299792458.0
-    return adv / grid.dt_u > line * traj.n_s
+def _per_step(traj, n_hat, grid):
+    """Grid points per step of the mean advance, averaged over the pixels of each tile of 512."""
+    span = _span(traj).cpu().numpy()
+    adv = span[0] - (n_hat[:, 0] * span[1] + n_hat[:, 1] * span[2]
+                     - (1.0 - n_hat[:, 2]) * span[3]) / 299792458.0
+    return [float(adv[k:k + 512].mean()) / (grid.dt_u * traj.n_s) for k in range(0, len(adv), 512)]
 
 
-def _kernel_us(call):
-    """Device time of the walk's and of the search's launches in one call [us]."""
-    from torch.profiler import ProfilerActivity, profile
-    call()
-    torch.cuda.synchronize()
-    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+def _ms(call):
+    """Shortest of seven calls, by events on the stream."""
+    times = []
+    for _ in range(9):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
         call()
-        torch.cuda.synchronize()
-    seen = {e.key: e.self_device_time_total for e in prof.key_averages()}
-    if not any("deposit_mixed_kernel" in k for k in seen):
-        pytest.skip("no trace of the launches here")
-    return [sum(v for k, v in seen.items() if name in k)
-            for name in ("deposit_walk_kernel", "deposit_mixed_kernel")]
+        b.record()
+        b.synchronize()
+        times.append(a.elapsed_time(b))
+    return min(times[2:])
 
 
-def test_each_tile_has_one_launch():
-    """Pixels from the axis outwards: 1 - n.beta grows with the angle, so that with this grid the
-    first tiles are searched, the last is walked, and both launches have work; with eight times
-    the bins all are walked and the search's CTAs end at once; without the order there is no walk."""
-    tr = simple.transverse_oscillation(256, 3000, 1e-17, 0.999, 0.002, 97.0, seed=8)
+def test_dense_tiles_are_walked():
+    """Pixels from the axis outwards: 1 - n.beta grows with the angle, and with it the grid points
+    per step of the three tiles (0.9, 1.6 and 3).  The first is searched, the others are walked:
+    seen by the time, which is longer when the stored mean advance says that no tile is dense (1.5, 3
+    points per step take about 0.6 and 0.5 of the search's time walked), and about the same as
+    that when the view's order stands elsewhere."""
+    tr = simple.transverse_oscillation(512, 3000, 1e-17, 0.999, 0.002, 97.0, seed=8)
     th = np.linspace(0.0, 0.09, 1536)
     n_hat = np.stack([np.sin(th), np.zeros_like(th), np.cos(th)], -1)
     traj = lw.lw_trajectories_upload(tr.t, tr.r, tr.beta, tr.beta_dot)
     det = lw.Detector(n_hat)
-    grid = _grid(traj, det, 6120)
-    fine = lw.Grid(grid.t_min, grid.dt_u / 8.0, grid.n_bins * 8)
-    prec = lw.LW_MIXED_F32X4
-    some, all_ = _dense(traj, n_hat, grid, 1.0), _dense(traj, n_hat, fine, 1.0)
-    assert not some[0] and some[-1] and all_.all()
-    walk_some, search_some = _kernel_us(lambda: _deposit(traj, det, grid, prec))
-    walk_all, search_all = _kernel_us(lambda: _deposit(traj, det, fine, prec))
-    walk_none, search_none = _kernel_us(lambda: _deposit(_searched(traj), det, grid, prec))
-    assert walk_none == 0 and search_none > search_some > 3 * search_all
-    assert walk_all > 3 * search_all and walk_some > 3 * search_all
+    grid = _grid(traj, det, 12300)
+    assert [v > 1.0 for v in _per_step(traj, n_hat, grid)] == [False, True, True]
+    rec, _ = _deposit(traj, det, grid, lw.LW_MIXED_F32X4)
+    walked, first = _ms(lambda: _deposit(traj, det, grid, lw.LW_MIXED_F32X4)), rec.clone()
+    other = _searched(traj)
+    moved = _ms(lambda: _deposit(other, det, grid, lw.LW_MIXED_F32X4))
+    _span(traj).zero_()
+    assert _per_step(traj, n_hat, grid) == [0.0, 0.0, 0.0]
+    searched = _ms(lambda: _deposit(traj, det, grid, lw.LW_MIXED_F32X4))
+    assert walked < 0.8 * searched and walked < 0.8 * moved
+    rec, _ = _deposit(traj, det, grid, lw.LW_MIXED_F32X4)
+    # FP32 additions of the same contributions in two orders; a tile deposited by both launches or by
+    # neither is an error of order one
+    assert (first - rec).abs().max() <= 1e-3 * rec.abs().max()
+
+
+@pytest.mark.parametrize("prec,per_step", [(lw.LW_MIXED_F32X4, 1.1), (lw.LW_MIXED_F32, 1.5),
+                                           (lw.LW_MIXED, 1.9), (lw.LW_MIXED_KAHAN, 4.3),
+                                           (lw.LW_MIXED_KAHAN, 8.0)])
+def test_a_bunch_is_not_slower_than_by_search(prec, per_step):
+    """Electrons of a bunch, each over its own part of the grid, just above the lines and beyond (grid
+    points per step, averaged over the 256 pixels)."""
+    w = configs.c2x(n_e=400, n_s=6000, nx=16, n_bins=1 << 12)
+    traj = lw.lw_trajectories_upload(w.traj.t, w.traj.r, w.traj.beta, w.traj.beta_dot)
+    other = _searched(traj)
+    det = lw.Detector(w.n_hat)
+    lo, hi = lw.lw_grid_bounds(traj, det).cpu().tolist()
+    grid = lw.grid_from_bounds(lo, hi, 1 << 16)
+    (had,) = _per_step(traj, w.n_hat, grid)
+    grid = lw.grid_from_bounds(lo, hi, int(per_step / had * (1 << 16)))
+    chosen = _ms(lambda: lw.lw_deposit_time_domain(traj, det, grid, prec))
+    searched = _ms(lambda: lw.lw_deposit_time_domain(other, det, grid, prec))
+    assert chosen <= 1.04 * searched
