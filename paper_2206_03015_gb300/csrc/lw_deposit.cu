@@ -69,6 +69,13 @@ struct DepositArgs {
     const double* span;   // mixed: mean advance, or null where no tile can be dense (walk_tile)
 };
 
+// Inputs whose advanced time need not increase from sample to sample: flagged by the upload (a step
+// longer than c0 dt, times out of order, non-finite values), or not known.
+__device__ __forceinline__ bool irregular(const DepositArgs& p) {
+    return !p.input_status ||
+           (*p.input_status & (LW_ST_STEP | LW_ST_TIME | LW_ST_NONFINITE)) != 0;
+}
+
 // ------------------------------------------------------------------ FP64
 
 constexpr int kFp64Threads = 128;
@@ -755,8 +762,8 @@ __device__ __noinline__ bool walk_tile(const double* span, const double* n_hat, 
 // The blocks of every electron may be divided over `parts` CTAs (part = 0 .. parts-1): a part
 // starts from its first block's anchor, whose bin is the end of the part before (the same
 // anchor, the same arithmetic).  Problems whose tiles and chunks are few fill the GPU that way.
-// Flagged inputs (a step longer than c0 dt, times out of order, non-finite values) are left to
-// part 0, where the last grid point reached is carried over the whole trajectory.
+// Irregular inputs are left to part 0, where the last grid point reached is carried over the whole
+// trajectory.
 //
 // With CHECK the CTAs of a unit (its parts, and with PIX = 1 the two halves of its tile) are a
 // cluster over which the unit's sums are taken.  Without SPLIT
@@ -826,7 +833,7 @@ __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int
     }
     __syncthreads();   // barriers initialised
     int bits = 0;
-    const int flagged = SPLIT && p.input_status ? *p.input_status : 0;
+    const bool whole = SPLIT && irregular(p);
     if (tile == 0 && chunk == 0 && part == 0 && threadIdx.x == 0 && p.input_status)
         bits |= *p.input_status;
     float err2 = 0.0f, val2 = 0.0f;   // CHECK: squared error estimates and squared values
@@ -843,7 +850,7 @@ __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int
     // whose end anchor is in the next one
     auto cut = [&](int q) -> int {
         if (!SPLIT) return q == 0 ? 0 : nbs;
-        if (flagged & (LW_ST_STEP | LW_ST_TIME | LW_ST_NONFINITE)) return q == 0 ? 0 : nbs;
+        if (whole) return q == 0 ? 0 : nbs;
         const int c = (int)((int64_t)nbs * q / parts);
         return c < nbs && (c & (kAnchorBatch - 1)) == kAnchorBatch - 1 ? c + 1 : c;
     };
@@ -1451,11 +1458,12 @@ __global__ void __launch_bounds__(kFp64Threads) deposit_fp64_kernel(DepositArgs 
     block_status_or(p.status, bits);
 }
 
-// walk_tile for the CTA (thread 0 decides)
+// walk_tile for the CTA (thread 0 decides).  Irregular inputs are searched: where coordinates go back
+// within a block, the walk's running maximum and the search's bisection can end in different steps.
 template <int ACC>
 __device__ __forceinline__ bool tile_is_dense(const DepositArgs& p, int64_t pix0) {
     int dense = 0;
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0 && !irregular(p))
         dense = walk_tile(p.span, p.n_hat, p.n_pix, pix0 / kWalkTile * kWalkTile + kWalkTile / 2,
                           walk_density<ACC>() * (double)(p.ns1 - 1), p.inv_dtu);
     return __syncthreads_or(dense) != 0;

@@ -55,6 +55,42 @@ def test_walk_and_search_agree_to_the_bit(prec, flags, n_s, per_step, block):
     assert walked.abs().max() > 0
 
 
+def _irregular(kind, n_e=1, n_s=600):
+    """Trajectories that the upload flags, from sample 250 of electron 0 on: a superluminal step (the
+    advanced time goes back by about 20 steps), a step backwards longer than c0 dt (over the rest
+    of the grid), a repeated sample, a sample whose time goes back, one
+    that is not finite."""
+    tr = simple.transverse_oscillation(n_e, n_s, 1e-17, 0.999, 0.01, 97.0, seed=6)
+    t, r = np.tile(tr.t, (n_e, 1)), tr.r.copy()
+    if kind == "back":
+        r[0, 250:, 2] += 9e-11
+    elif kind == "ahead":
+        r[0, 250:, 2] -= 6.2e-9
+    elif kind == "repeat":
+        t[0, 250], r[0, 250] = t[0, 249], r[0, 249]
+    elif kind == "time":
+        t[0, 250] -= 2.5e-17
+    else:
+        r[0, 250, 0] = np.nan
+    return simple.Trajectories(t, r, tr.beta, tr.beta_dot)
+
+
+@pytest.mark.parametrize("prec", [lw.LW_MIXED, lw.LW_MIXED_F32, lw.LW_MIXED_F32X4])
+@pytest.mark.parametrize("kind", ["back", "ahead", "repeat", "time", "nan"])
+def test_irregular_inputs_are_searched(prec, kind):
+    """Dense tiles of inputs that the upload flags: the record and the status of the search, also
+    where the coordinate goes back within a block."""
+    clean = simple.transverse_oscillation(1, 600, 1e-17, 0.999, 0.01, 97.0, seed=6)
+    det = lw.Detector(_n_hat(70))
+    grid = _grid(lw.lw_trajectories_upload(clean.t, clean.r, clean.beta, clean.beta_dot), det, 3000)
+    tr = _irregular(kind)
+    traj = lw.lw_trajectories_upload(tr.t, tr.r, tr.beta, tr.beta_dot, block=512)
+    got, st = _deposit(traj, det, grid, prec)
+    want, st_s = _deposit(_searched(traj), det, grid, prec)
+    assert st == st_s and st & (lw.LW_ST_STEP | lw.LW_ST_TIME | lw.LW_ST_NONFINITE)
+    assert torch.equal(got, want) and bool(torch.isfinite(got).all()) and got.abs().max() > 0
+
+
 def _span(traj):
     """The mean advance that the upload stores behind the order: after two keys and 4,096 counters."""
     at = traj.view.order + (4 * traj.n_e + 255) // 256 * 256 + 16 + 4 * 4096 - traj.ws.data_ptr()
