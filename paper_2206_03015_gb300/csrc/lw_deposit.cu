@@ -79,7 +79,6 @@ __device__ __forceinline__ bool irregular(const DepositArgs& p) {
 // ------------------------------------------------------------------ FP64
 
 constexpr int kFp64Threads = 128;
-constexpr int kFp64Tile = 64;
 
 // FP64 instructions are what these kernels pay for (GB300: 19 cycles per warp instruction and
 // SM), so quotients with a common divisor share its correctly rounded reciprocal r: with one
@@ -230,51 +229,6 @@ __device__ __forceinline__ void scan_sample(const DepositArgs& p, double nx, dou
     S.tb = ta;
     S.ub = ua;
     S.ok_b = ok_a;
-}
-
-// Algorithm 2 literally: every step of every (pixel, electron), in the oracle's
-// operation order (CTA = kFp64Threads pixels x p.e_chunk electrons).
-__device__ void fp64_scan_cta(const DepositArgs& p) {
-    __shared__ double s_t[kFp64Tile];
-    __shared__ double s_r[kFp64Tile * 3];
-    const int64_t m = (int64_t)blockIdx.x * kFp64Threads + threadIdx.x;
-    const bool active = m < p.n_pix;
-    double nx = 0.0, ny = 0.0, nz = 1.0;
-    if (active) {
-        nx = p.n_hat[3 * m];
-        ny = p.n_hat[3 * m + 1];
-        nz = p.n_hat[3 * m + 2];
-    }
-    double* rec = static_cast<double*>(p.record) + (active ? m * 3 * p.n_bins : 0);
-    int bits = 0;
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && p.input_status)
-        bits |= *p.input_status;
-    const int64_t k0 = (int64_t)blockIdx.y * p.e_chunk;
-    const int64_t k1 = min(k0 + p.e_chunk, p.n_e);
-    for (int64_t k = k0; k < k1; ++k) {
-        const double* tk = p.t + (p.t_per_e ? k * p.ns1 : 0);
-        const double* rk = p.r + 3 * k * p.ns1;
-        const double* bk = p.beta + 3 * k * p.ns1;
-        const double* ak = p.bdot + 3 * k * p.ns1;
-        ScanState S;
-        S.reset();
-        for (int64_t i0 = 0; i0 < p.ns1; i0 += kFp64Tile) {
-            const int n = (int)min((int64_t)kFp64Tile, p.ns1 - i0);
-            __syncthreads();
-            for (int q = threadIdx.x; q < n; q += kFp64Threads) {
-                s_t[q] = tk[i0 + q];
-                s_r[3 * q] = rk[3 * (i0 + q)];
-                s_r[3 * q + 1] = rk[3 * (i0 + q) + 1];
-                s_r[3 * q + 2] = rk[3 * (i0 + q) + 2];
-            }
-            __syncthreads();
-            if (!active) continue;
-            for (int q = 0; q < n; ++q)
-                scan_sample(p, nx, ny, nz, rec, bk, ak, i0 + q, s_t[q], s_r[3 * q],
-                            s_r[3 * q + 1], s_r[3 * q + 2], S, bits);
-        }
-    }
-    block_status_or(p.status, bits);
 }
 
 // ------------------------------------------------------------------ mixed
@@ -1269,8 +1223,10 @@ __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int
 //  * more than half a grid point per step on average: every step in order from staged blocks,
 //    fields once per step (64 electrons x 1,200 steps x 400 pixels x 4,096 bins, 3.4 points
 //    per step: 17.0 ms before the shared reciprocals and the division over grid z, now 9.0).
-// Inputs that the upload flagged (a step longer than c0 dt, times out of order, non-finite
-// values) take the literal scan.
+// The latter is Algorithm 2 literally and takes every electron whose advanced time need not increase:
+// of irregular inputs a CTA tests each electron's samples, so that one bad sample costs its electron
+// only (one of 1,000 electrons x 5,000 steps x 1,024 pixels: 6.5 ms beside 1.7 without; 156 with
+// all of them taken step by step).
 constexpr int kF64Block = 64;   // samples staged per block
 
 // The first of the samples 1 .. last whose coordinate reaches j, by the scan's FP64 coordinate alone
@@ -1302,11 +1258,19 @@ __device__ __noinline__ int first_sample_fp64(const double* n, const double* r, 
     return ib;
 }
 
-__global__ void __launch_bounds__(kFp64Threads) deposit_fp64_kernel(DepositArgs p) {
-    if (p.input_status && (*p.input_status & (LW_ST_STEP | LW_ST_TIME | LW_ST_NONFINITE))) {
-        if (blockIdx.z == 0) fp64_scan_cta(p);
-        return;
+// Whether the thread's share of an electron's steps is subluminal and forward in time, as the upload
+// tests them (out of line: irregular inputs only).
+__device__ __noinline__ bool steps_in_order(const double* r, const double* t, int last) {
+    for (int i = 1 + (int)threadIdx.x; i <= last; i += kFp64Threads) {
+        const double* x = r + 3 * (int64_t)i;
+        const double dx = x[0] - x[-3], dy = x[1] - x[-2], dz = x[2] - x[-1];
+        const double dt = t[i] - t[i - 1], ct = kC0 * dt;
+        if (!(dt > 0.0) || !(dx * dx + dy * dy + dz * dz < ct * ct)) return false;
     }
+    return true;
+}
+
+__global__ void __launch_bounds__(kFp64Threads) deposit_fp64_kernel(DepositArgs p) {
     __shared__ double s_t[2][kF64Block + 1];        // sample i0-1 first
     __shared__ double s_r[2][3 * (kF64Block + 1)];
     __shared__ double s_n[kFp64Threads][3];         // pixel directions
@@ -1341,6 +1305,7 @@ __global__ void __launch_bounds__(kFp64Threads) deposit_fp64_kernel(DepositArgs 
     if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0 &&
         p.input_status)
         bits |= *p.input_status;
+    const bool flagged = irregular(p);
     const int nblk = (int)((p.ns1 + kF64Block - 1) / kF64Block);
     auto coord = [&](double ta) { return __dmul_rn(__dsub_rn(ta, p.t_min), p.inv_dtu); };
     const int64_t k0 = (int64_t)blockIdx.y * p.e_chunk;
@@ -1355,6 +1320,7 @@ __global__ void __launch_bounds__(kFp64Threads) deposit_fp64_kernel(DepositArgs 
         const double u0 = coord(advanced_time_fp64(nx, ny, nz, e0[1], e0[2], e0[3], e0[0]));
         const double ul = coord(advanced_time_fp64(nx, ny, nz, e0[5], e0[6], e0[7], e0[4]));
         const bool ok = in_range(u0) && in_range(ul);
+        const bool in_order = (!active || ok) && (!flagged || steps_in_order(rk, tk, last));
         int64_t a = 0, z = -1;   // the pixel's run
         if (active && ok) {
             a = __double2ll_rd(u0) + 1;
@@ -1376,7 +1342,7 @@ __global__ void __launch_bounds__(kFp64Threads) deposit_fp64_kernel(DepositArgs 
         s_ja[threadIdx.x] = (int)a;
         s_u[threadIdx.x][0] = u0;
         s_u[threadIdx.x][1] = ul;
-        const int bad = __syncthreads_or(active && !ok);
+        const int bad = __syncthreads_or(!in_order);
         long long before = 0, T = 0;
         for (int w = 0; w < kFp64Threads / 32; ++w) {
             if (w < warp) before += s_warp[w];
