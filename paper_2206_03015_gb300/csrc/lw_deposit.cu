@@ -83,14 +83,22 @@ constexpr int kFp64Threads = 128;
 // FP64 instructions are what these kernels pay for (GB300: 19 cycles per warp instruction and
 // SM), so quotients with a common divisor share its correctly rounded reciprocal r: with one
 // residual correction n r is the correctly rounded quotient (Markstein), 3 instructions after
-// the 5 of the reciprocal instead of 8 per division.  Where the product or the correction
-// leaves the finite range the division itself decides
-// (a call, so that its instructions are not issued beside the common path under a predicate).
+// the 5 of the reciprocal instead of 8 per division.  The residual n - q d is exact while n and q
+// are 2^-960 or more in size (d below 2^1022), so outside that range the division itself decides
+// (a call, so that its instructions are not issued beside the common path under a predicate);
+// zeros, the field where nothing accelerates, keep the product.  tests/test_rounding_model.py has
+// the same steps.
 __device__ __noinline__ double divide_rare(double n, double d) { return __ddiv_rn(n, d); }
 __device__ __forceinline__ double quotient(double n, double d, double r) {
-    double q = __dmul_rn(n, r);
-    q = __fma_rn(__fma_rn(-q, d, n), r, q);
-    if ((__double2hiint(q) & 0x7ff00000) == 0x7ff00000) q = divide_rare(n, d);
+    constexpr unsigned kLeast = (1023u - 960u) << 20, kInf = 0x7ff00000u;
+    const double q0 = __dmul_rn(n, r);
+    const double q = __fma_rn(__fma_rn(-q0, d, n), r, q0);
+    const unsigned hn = __double2hiint(n) & 0x7fffffff, hq = __double2hiint(q) & 0x7fffffff;
+    if (hn < kLeast || hq - kLeast >= kInf - kLeast) {
+        const bool zero = (hn | __double2loint(n) | (__double2hiint(q0) & 0x7fffffff) |
+                           __double2loint(q0)) == 0;
+        return zero ? q0 : divide_rare(n, d);
+    }
     return q;
 }
 // x > 0 and |x| < 2^62 on the bits (integer pipe; NaN and infinities fail)
