@@ -82,15 +82,17 @@ __device__ __forceinline__ BeamValue beam_value(const Beam& B, double x, double 
 }
 __device__ __forceinline__ double beam_unit(const BeamValue& b) { return b.A * fma(b.s, b.sn, b.cs); }
 
-// n / d correctly rounded, given the reciprocal r of d to an ulp (residual correction; the
-// error left before the last rounding is 2^-105 of the quotient)
+// n / d rounded as the division rounds it, given the reciprocal r of d to an ulp: residual correction
+// (Markstein), exact while n and the quotient are above 2^-960 in size, 2^-105 of the quotient before
+// the last rounding.  Below that (a momentum component of 1e-289) last bits of the quotient differ.
 __device__ __forceinline__ double quotient(double n, double d, double r) {
     const double q = __dmul_rn(n, r);
     return fma(fma(-q, d, n), r, q);
 }
 
-// gamma = sqrt(a), correctly rounded, and its reciprocal to an ulp (a = 1 + u^2 >= 1; an
-// infinite or NaN a ends as NaN)
+// gamma = sqrt(a), rounded as the square root rounds it, and its reciprocal to an ulp (a = 1 + u^2 >= 1;
+// an infinite or NaN a ends as NaN): residual correction from a reciprocal root good to an ulp
+// (Markstein; tests/test_rounding_model.py has its steps)
 __device__ __forceinline__ double root(double a, double& inv) {
     const double y = rsqrt(a);
     const double g = __dmul_rn(a, y);
@@ -542,7 +544,9 @@ Laser laser_constants(const lw_laser& l) {
     L.k = L.omega * kInvC0;
     L.sigma = l.fwhm / (2.0 * sqrt(log(2.0)));
     L.E0 = l.a0 * kMe * kC0 * L.omega / kQe;
-    L.zR = kPi * l.w0 * l.w0 / l.lam;
+    // finite, so that zeta/zR by its reciprocal is (a plane wave given as a huge waist; the product
+    // overflows from w0 = 1e151 on): at 1e300 zeta/zR and its square add nothing
+    L.zR = fmin(kPi * l.w0 * l.w0 / l.lam, 1.0e300);
     L.w0 = l.w0;
     return L;
 }
