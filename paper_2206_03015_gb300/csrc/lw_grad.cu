@@ -188,7 +188,8 @@ __device__ __forceinline__ void sample_field(double nx, double ny, double nz,
     // the forward's D to the bit: 1e-16 of rounding in n . beta is 1e-12 of D at gamma 60
     const double D = __dsub_rn(1.0, __dadd_rn(__dadd_rn(__dmul_rn(nx, b0), __dmul_rn(ny, b1)),
                                               __dmul_rn(nz, b2)));
-    const bool ok = fma(b2, b2, fma(b1, b1, b0 * b0)) < 1.0 && D > 0.0;
+    // the forward's test too: a sample whose field it takes as zero has no gradient
+    const bool ok = D > 0.0 && subluminal(b0, b1, b2);
     f.iD = ok ? __drcp_rn(D) : 0.0;
     f.iD3 = f.iD * f.iD * f.iD;
     for (int c = 0; c < 3; ++c) f.F[c] = fma(f.m[c], f.k, -f.a[c] * f.nm) * f.iD3;

@@ -118,6 +118,20 @@ __device__ __forceinline__ float to_float(double v) {
     return to_float_bits((unsigned)__double2hiint(v), (unsigned)__double2loint(v));
 }
 
+// |beta|^2 < 1, decided in FP32 where 1 - beta^2 is far above its FP32 rounding (as in the
+// upload), else by the FP64 expression ((bx*bx + by*by) + bz*bz) < 1
+static __device__ __noinline__ bool subluminal_exact(double b0, double b1, double b2) {
+    return __dadd_rn(__dadd_rn(__dmul_rn(b0, b0), __dmul_rn(b1, b1)), __dmul_rn(b2, b2)) < 1.0;
+}
+__device__ __forceinline__ bool subluminal(double b0, double b1, double b2) {
+    const float eps = to_float(1.0 - b2);
+    const float x = to_float(b0), y = to_float(b1);
+    const float perp = fmaf(x, x, y * y);
+    const float one_minus = fmaf(-eps, eps, 2.0f * eps) - perp;
+    if (__double2hiint(b2) >= 0x3fe00000 && one_minus > 1.0e-5f * (2.0f * eps + perp)) return true;
+    return subluminal_exact(b0, b1, b2);
+}
+
 // Far-field advanced time t_a = t - (n . r) / c0 in FP64 with the documented
 // operation order ((n_x x + n_y y) + n_z z), one rounding per operation.
 __device__ __forceinline__ double advanced_time_fp64(double nx, double ny, double nz, double x,
