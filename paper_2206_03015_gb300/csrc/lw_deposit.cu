@@ -594,19 +594,19 @@ struct WalkStage {
 };
 static_assert(sizeof(WalkStage) <= sizeof(int2) * kJobTable, "a warp's walk lies in its job table");
 
-template <int PIX, int ACC, int FL>
+template <int ACC, int FL>
 __device__ __forceinline__ void walk_block(const float4* s_scan, const float4* s_f4,
-                                        const float2* s_f2, int ns, const float4* s_wh,
-                                        const int4* s_job, int2 K2, int2 JA2, float s32,
-                                        float inv_sc, float c0_over_R, int64_t n_bins,
-                                        unsigned char* tile_rec, WalkStage& st) {
+                                           const float2* s_f2, int ns, const float4* s_wh,
+                                           const int4* s_job, int K_lane, int ja_lane, float s32,
+                                           float inv_sc, float c0_over_R, int64_t n_bins,
+                                           unsigned char* tile_rec, WalkStage& st) {
     const int lane = threadIdx.x & 31;
     const uint64_t row_bytes =
         4ull * (ACC == kAccF32X4 ? 4 : ACC == kAccF32 ? 3 : 6) * (uint64_t)n_bins;
-    for (int slot = 0; slot < 32 * PIX; ++slot) {   // s_wh, s_job: the warp's slots
-        const int K = __shfl_sync(0xffffffffu, slot % PIX ? K2.y : K2.x, slot / PIX);
+    for (int slot = 0; slot < 32; ++slot) {   // s_wh, s_job: the warp's slots, one per lane
+        const int K = __shfl_sync(0xffffffffu, K_lane, slot);
         if (K == 0) continue;
-        const int ja = __shfl_sync(0xffffffffu, slot % PIX ? JA2.y : JA2.x, slot / PIX);
+        const int ja = __shfl_sync(0xffffffffu, ja_lane, slot);
         const int4 jb = s_job[slot];
         const float4 w = s_wh[slot];
         const float f = __int_as_float(jb.y), xe = __int_as_float(jb.z);
@@ -1001,13 +1001,11 @@ __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int
                 fs[q] = fe;
             }
             if constexpr (MODE == kWalk) {
-                for (int q = 0; q < PIX; ++q) K[q] += big[q];
+                static_assert(PIX == 1, "one pixel per lane");
                 __syncwarp();   // the warp's slot records are written
-                walk_block<PIX, ACC, FL>(
-                    s_scan, s_f4, s_f2, ns, s_wh + wslot, s_job + wslot,
-                    make_int2(K[0], K[PIX - 1]), make_int2(JA[0], JA[PIX - 1]), s32, inv_sc,
-                    c0_over_R, p.n_bins, tile_rec,
-                    *reinterpret_cast<WalkStage*>(&s_tab[warp][0]));
+                walk_block<ACC, FL>(s_scan, s_f4, s_f2, ns, s_wh + wslot, s_job + wslot,
+                                    K[0] + big[0], JA[0], s32, inv_sc, c0_over_R, p.n_bins,
+                                    tile_rec, *reinterpret_cast<WalkStage*>(&s_tab[warp][0]));
                 continue;
             }
             // Grid point j (absolute) of slot sl with block data I, f, xe (coordinate of the

@@ -647,12 +647,7 @@ int run_spectrum(const void* record, int kind, int64_t n_pix, const lw_grid* g, 
     if (direct) {
         if (cudaMemsetAsync(S, 0, sizeof(T) * (size_t)nl * (size_t)n_pix, st) != cudaSuccess)
             return LW_ECUDA;
-        const size_t smem = sizeof(C) * (size_t)fft_slots((int)N, logN, 1);
-        if (smem > 48 * 1024 &&
-            cudaFuncSetAttribute(spectrum_direct_kernel<T>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem) != cudaSuccess)
-            return LW_ECUDA;
+        const size_t smem = sizeof(C) * (size_t)fft_slots((int)N, logN, 1);   // 8.5 KB at most
         spectrum_direct_kernel<T><<<(unsigned)n_pairs, 256, smem, st>>>(
             rd, n_pix, (int)N, logN, scale, tw, S, X);
         return launch_status();
