@@ -540,12 +540,10 @@ def run_ours(args, rank, world, dist):
 
     # launches of our kernels per timed step: upload (prepare, and ends and electron order in
     # one launch up to 2,048 electrons, else ends, key init, range, count, scan, scatter),
-    # deposit (search, precision check, and the walk of dense tiles where the grid can hold
-    # as many points per step as the record's line says), spectrum (twiddle and one transform
+    # deposit (the deposit and its precision check), spectrum (twiddle and one transform
     # kernel, or the two passes above 16,384 bins and above 4,096 with fewer than 76 pixel pairs)
     upload_k = 2 if tr.n_e <= 2048 else 7
-    line = {lw.LW_MIXED_F32X4: 1.0, lw.LW_MIXED_F32: 1.4}.get(MIX, 1.8)
-    deposit_k = 3 if grid.n_bins > line * tr.n_s else 2
+    deposit_k = 2
     spec_k = 2 if grid.n_bins <= 4096 or (grid.n_bins <= 16384 and det.n_pix > 150) else 3
     result["gpu_launches"] = args.steps * (upload_k + deposit_k + spec_k)
     if rank == 0 and world == 1 and not args.no_cpu_baseline:

@@ -1,27 +1,30 @@
 // Time-domain deposit (Algorithm 2 of the paper) for every pixel.
 //
-// Thread mapping (both precisions): one thread owns one (mixed: PIX) detector
-// pixel(s) -- the paper's "detector parallelization" on one GPU -- and a CTA
-// walks a chunk of electrons; the samples of the current electron are staged
-// in shared memory once per CTA and read by all of its pixels as broadcasts.
-// The field (Eq. far_efield) and the interpolation weights are evaluated only
-// for steps whose interval (t_b, t_a] contains grid points, and those
-// contributions are added to the record with global atomics (pixels of
-// different CTAs share bins through electrons of other chunks).
+// A CTA owns a tile of detector pixels -- the paper's "detector parallelization"
+// on one GPU -- and a chunk of electrons.  The field (Eq. far_efield) and the
+// interpolation weights are evaluated only for steps whose interval (t_b, t_a]
+// contains grid points, and those contributions are added to the record with
+// global atomics (CTAs share bins through electrons of other chunks).
 //
-// FP64 path (deposit_fp64_kernel): every result of the time map, the bin index,
+// FP64 path (deposit_fp64_kernel): where grid points are few the tile's points of
+// an electron are listed and taken one per thread, each searching its step among
+// the stored samples; where they are many, and for trajectories out of order, a
+// thread owns a pixel and takes every step from staged blocks of samples.  Every
+// result of the time map, the bin index,
 // the field and the weights is the correctly rounded one of the operation order
 // documented in lw.h, so advanced times, bin indices and per-sample contributions
 // are bit-identical to a plain C loop without FMA contraction; only the order of
 // the atomic additions differs.
 //
-// Mixed path: the bin coordinate u = (t_a - t_min)/dt_u is anchored once per
+// Mixed path: a thread owns one or two pixels and the electron's samples are staged
+// block by block in shared memory, once per CTA.  The bin coordinate u = (t_a - t_min)/dt_u is anchored once per
 // block of samples in double-FP32 arithmetic (integer part + FP32 fraction)
 // and evaluated per sample with three FP32 FMAs of small, block-relative
 // quantities.  Because t_a increases along a subluminal trajectory, a block
 // needs one coordinate per pixel (its last sample) to know which grid points
 // it reaches; each grid point's step is then found by a bracketed search
-// (regula falsi, then bisection) over the staged block.  The field is FP32 in
+// (regula falsi, then bisection) over the staged block, or, where grid points are as
+// many as steps, the block is walked sample by sample.  The field is FP32 in
 // the stable form
 //   D = (1 - n_z) + n_z (1 - beta_z) - n_perp . beta_perp,
 // and contributions are added with FP64 atomics, a compensated pair of FP32
@@ -565,22 +568,22 @@ __device__ __forceinline__ int frac_floor(float f) { return f >= 1.0f ? 1 : (f <
 // run's bounds ja .. ja + K - 1 go to the first and the last step).
 // A contribution is the search's to the bit: the samples keep their end terms and scale apart (five
 // words), and a grid point weights and sums them in the search's operations.  Interpolating between
-// fields already multiplied out (four words, 6 % faster: 17.4 and 18.6 ms below) rounds otherwise and
-// moved a gradient over 2,048 electrons, which adds up what they share.
+// fields already multiplied out (four words, 6 % faster) rounds otherwise and moved a gradient over
+// 2,048 electrons, which adds up what they share.
 // 512 co-located electrons x 4,096 steps x 1,024 pixels, search and walk at 1.05, 1.5 and 3 grid
-// points per step: interleaved FP32 record 18.9 and 18.6, 24.6 and 18.8, 48 and 23 ms; FP32 rows
-// (1.45, 2) 27.0 and 26.0, 33 and 23; FP64 record (1.85, 2, 3) 38 and 35, 37 and 28, 56 and 47.
+// points per step: interleaved FP32 record 18.8 and 21.8, 24.4 and 22.0, 48 and 26 ms; FP32 rows
+// (1.45, 2) 27.0 and 28.3, 33 and 25; FP64 record (1.85, 2, 3) 38.8 and 39.3, 38 and 32, 58 and 49.
 // The line lies where the walk gains on electrons that start together; those of a bunch gain earlier
-// (1,000 electrons x 10,000 steps x 256 pixels: interleaved record at 1.05 44 and 27, FP32 rows at
-// 1.45 63 and 38, FP64 record at 1.85 92 and 65 ms).  The compensated record is always searched: its
+// (1,000 electrons x 10,000 steps x 256 pixels: interleaved record at 1.05 43 and 29, FP32 rows at
+// 1.45 63 and 39, FP64 record at 1.85 95 and 63 ms).  The compensated record is always searched: its
 // returning additions of neighbouring grid points, which the walk puts side by side, wait for one
 // another (4.1, 6 and 10 points per step: the 512 electrons 118 and 101, 164 and 131, 288 and 223 ms,
 // but the bunch 356 and 386, 522 and 551; 400 electrons of it 75 and 87, 105 and 117, 175 and 193).
 // 2,048 co-located electrons x 4,096 steps x 1,024 pixels x 16,384 bins (1 to 5 grid points per
-// step): 238 ms by search, 83 ms walked.
+// step): 238 ms by search, 89 ms walked.
 template <int ACC>
-__host__ __device__ constexpr double walk_density() {
-    return ACC == kAccF32X4 ? 1.0 : ACC == kAccF32 ? 1.4 : 1.8;
+__host__ __device__ constexpr float walk_density() {
+    return ACC == kAccF32X4 ? 1.3f : ACC == kAccF32 ? 1.6f : 1.9f;
 }
 constexpr int kWalkTile = 512;  // pixels that share a decision
 constexpr int kWalkMap = 256;   // grid points of a segment mapped to steps at a time
@@ -676,10 +679,9 @@ __device__ __forceinline__ void walk_block(const float4* s_scan, const float4* s
 }
 
 // Whether the electrons are walked for the 512 pixels around `pix`: the grid points per step that
-// the trajectories' mean advance (span, stored by the upload) gives the middle pixel.  Two launches
-// share a deposit's tiles by this test, so it is one function (out of line) of the call's arguments
-// only.  A test of every electron, by each of the search's CTAs, cost more than it sorted out
-// (36 FP64 instructions: 10 % of a 1,001-electron step).
+// the trajectories' mean advance (span, stored by the upload) gives the middle pixel.  A test of
+// every electron, by each CTA, cost more than it sorted out (36 FP64 instructions: 10 % of a
+// 1,001-electron step).
 __device__ __noinline__ bool walk_tile(const double* span, const double* n_hat, int64_t n_pix,
                                        int64_t pix, double points, double inv_dtu) {
     const double* n = n_hat + 3 * min(pix, n_pix - 1);
@@ -719,6 +721,19 @@ __device__ __noinline__ bool walk_tile(const double* span, const double* n_hat, 
 // (one part, known at compile time) the deposit keeps the registers that the parts cost it
 // (80 instead of 74 with spills: 0.8 % of a 10,000-electron step).
 enum { kSearch = 0, kWalk = 1, kCheck = 2 };   // deposit by search, by walk, or check
+struct MixShared {   // a CTA's slots and tables
+    float4 wh[kMixThreads * kMixPix];   // slope hi parts (w_x, w_y, w_z), row
+    int4 job[kMixThreads * kMixPix];    // block: I, f, x_end
+    int ja[kMixThreads * kMixPix];      // block: first grid point
+    int kp[kMixThreads * kMixPix];      // block: job offset (lane-major)
+    int2 tab[kMixThreads / 32][kJobTable];   // block: (slot, grid point) of job t
+    uint64_t full[kMixStages];               // stage filled (bytes arrived)
+};
+// (one object for the search and the walk of a kernel that has both)
+__device__ __forceinline__ MixShared& mix_shared() {
+    __shared__ __align__(16) MixShared sh;
+    return sh;
+}
 template <int PIX, int ACC, int FL, int MODE, bool SPLIT>
 __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int64_t chunk,
                                          int part_ = 0, int parts_ = 1) {
@@ -732,12 +747,13 @@ __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int
     // Slot numbering: lane-major, wslot + lane * PIX + q for pixel q of a lane -- the
     // order in which the warp's jobs are listed, so that the 32 jobs of a round, which
     // mostly belong to consecutive slots, read consecutive per-slot records.
-    __shared__ float4 s_wh[kSlots];                   // slope hi parts (w_x, w_y, w_z), row
-    __shared__ int4 s_job[kSlots];                    // block: I, f, x_end
-    __shared__ int s_ja[kSlots];                      // block: first grid point
-    __shared__ int s_kp[kSlots];                      // block: job offset (lane-major)
-    __shared__ __align__(16) int2 s_tab[kWarpsMix][kJobTable];   // block: (slot, grid point) of job t
-    __shared__ __align__(8) uint64_t s_full[kMixStages];   // stage filled (bytes arrived)
+    MixShared& sh = mix_shared();
+    float4* const s_wh = sh.wh;
+    int4* const s_job = sh.job;
+    int* const s_ja = sh.ja;
+    int* const s_kp = sh.kp;
+    int2(*const s_tab)[kJobTable] = sh.tab;
+    uint64_t* const s_full = sh.full;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int wslot = warp * 32 * PIX;
@@ -1212,7 +1228,7 @@ __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int
 //    difference u - j in three FP64 instructions and FP32, confirms the two samples with
 //    the scan's coordinate and deposits.  Samples are read where the search lands, nothing is
 //    staged.  (A search per staged block of 256 samples left 5 of 32 lanes busy at 3 grid
-//    points per trajectory: 1,000 electrons x 5,000 steps x 1,024 pixels 7.9 ms, now 1.3 ms.)
+//    points per trajectory: 1,000 electrons x 5,000 steps x 1,024 pixels 8.0 ms, now 1.6 ms.)
 //  * more than half a grid point per step on average: every step in order from staged blocks,
 //    fields once per step (64 electrons x 1,200 steps x 400 pixels x 4,096 bins, 3.4 points
 //    per step: 17.0 ms before the shared reciprocals and the division over grid z, now 9.0).
@@ -1456,7 +1472,7 @@ __global__ void __launch_bounds__(kFp64Threads) deposit_fp64_kernel(DepositArgs 
     block_status_or(p.status, bits);
 }
 
-// walk_tile for the CTA (thread 0 decides).  Irregular inputs are searched: where coordinates go back
+// walk_tile for the CTA (thread 0 decides; out of line it keeps its registers).  Irregular inputs are searched: where coordinates go back
 // within a block, the walk's running maximum and the search's bisection can end in different steps.
 template <int ACC>
 __device__ __forceinline__ bool tile_is_dense(const DepositArgs& p, int64_t pix0) {
@@ -1472,20 +1488,27 @@ __global__ void __launch_bounds__(kMixThreads, kMixMinBlocks) deposit_mixed_kern
     // the precision check launched after this grid (programmatic dependent launch) may
     // start once every CTA of this grid has started: it fills the SMs of the last wave
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (ACC != kAccKahan && p.span && tile_is_dense<ACC>(p, (int64_t)blockIdx.x * (kMixThreads * PIX)))
-        return;
-    const int bits =
-        mixed_cta<PIX, ACC, FL, kSearch, SPLIT>(p, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.z);
-    block_status_or(p.status, bits);
-}
-
-// The tiles whose grid points are dense, walked (launched before the search; a launch without dense
-// tiles is about four waves of CTAs that end at once, 5 us).
-template <int ACC, int FL>
-__global__ void __launch_bounds__(kMixThreads, kMixMinBlocks) deposit_walk_kernel(DepositArgs p) {
-    if (!tile_is_dense<ACC>(p, (int64_t)blockIdx.x * kMixThreads)) return;
-    const int bits = mixed_cta<1, ACC, FL, kWalk, true>(p, blockIdx.x, blockIdx.y, blockIdx.z,
-                                                        gridDim.z);
+    int bits = 0;
+    if (ACC != kAccKahan && p.span &&
+        tile_is_dense<ACC>(p, (int64_t)blockIdx.x * (kMixThreads * PIX))) {
+        // One pixel per thread (two spill 36 to 210 bytes, 11 % slower): the tile's halves in turn.
+        // The same unit as the search's, so that electrons are added in the order in which they are
+        // searched: an FP32 record is rounded at every addition, and units of four electrons instead
+        // of one moved dL/dw0 of 2,048 electrons by 0.9 to 1.5 of its run-to-run deviations.  (Walked
+        // by a launch of its own, which does not run through one tile's halves in turn, that deposit
+        // takes 83 ms instead of 89; but where no tile is dense its CTAs all start only to end:
+        // 5 of 53 us of 226 electrons x 1,855 steps x 714 pixels, 9 of 850, 150 of 18,450.)
+#pragma unroll 1
+        for (int h = 0; h < PIX; ++h) {
+            const int64_t tile = (int64_t)blockIdx.x * PIX + h;
+            if (tile * kMixThreads < p.n_pix)
+                bits |= mixed_cta<1, ACC, FL, kWalk, SPLIT>(p, tile, blockIdx.y, blockIdx.z,
+                                                            gridDim.z);
+        }
+    } else {
+        bits = mixed_cta<PIX, ACC, FL, kSearch, SPLIT>(p, blockIdx.x, blockIdx.y, blockIdx.z,
+                                                       gridDim.z);
+    }
     block_status_or(p.status, bits);
 }
 
@@ -1590,15 +1613,6 @@ BatchedKernel batched_kernel_fl(uint32_t fl) {
     return fl == 1 ? deposit_batched_kernel<kMixPix, ACC, 1>
            : fl == 2 ? deposit_batched_kernel<kMixPix, ACC, 2>
                      : deposit_batched_kernel<kMixPix, ACC, 3>;
-}
-template <int ACC>
-MixedKernel walk_kernel_fl(uint32_t fl) {
-    return fl == 1 ? deposit_walk_kernel<ACC, 1>
-           : fl == 2 ? deposit_walk_kernel<ACC, 2> : deposit_walk_kernel<ACC, 3>;
-}
-MixedKernel walk_kernel(int acc, uint32_t fl) {
-    return acc == kAccF32 ? walk_kernel_fl<kAccF32>(fl)
-           : acc == kAccF32X4 ? walk_kernel_fl<kAccF32X4>(fl) : walk_kernel_fl<kAccF64>(fl);
 }
 using CheckKernel = void (*)(DepositArgs, int);
 template <int PIX, bool SPLIT>
@@ -1732,30 +1746,13 @@ extern "C" int lw_deposit_time_domain(const lw_traj* traj, const lw_detector* de
         g.z = (unsigned)std::min<int64_t>(std::min<int64_t>(nbs, 64), (two_waves + ctas - 1) / ctas);
     }
     const size_t smem = kMixStages * stage_bytes(traj->block);   // staging ring
-    // dense tiles (decided on the device, walk_tile) are walked by a launch of their own where the
-    // grid can hold that many points per step
+    // dense tiles (decided on the device, walk_tile) are walked, where the grid can hold that many
+    // points per step
     const int acc = acc_of(precision);
-    const double density = acc == kAccF32X4 ? walk_density<kAccF32X4>()
-                           : acc == kAccF32 ? walk_density<kAccF32>() : walk_density<kAccF64>();
-    if (acc != kAccKahan && (double)grid->n_bins > density * (double)traj->n_s)
+    const float density = acc == kAccF32X4 ? walk_density<kAccF32X4>()
+                          : acc == kAccF32 ? walk_density<kAccF32>() : walk_density<kAccF64>();
+    if (acc != kAccKahan && (double)grid->n_bins > (double)density * (double)traj->n_s)
         a.span = traj_span(traj);
-    if (a.span) {
-        // electrons in the search's chunks and order: an FP32 record is rounded at every addition,
-        // and chunks of four electrons instead of one moved dL/dw0 of 2,048 electrons by 0.9 to 1.5
-        // of its run-to-run deviations (now 0.2 to 0.6; chunks of two, or of four electrons as far
-        // apart as there are in flight: up to 1.9).  Where no tile is dense these CTAs, 9,009 in a
-        // 1,001-electron step of 840 us, end at once: 11 us, with four electrons in each 2.
-        const int64_t wx = (det->n_pix + kMixThreads - 1) / kMixThreads;
-        const int64_t chunks = (traj->n_e + a.e_chunk - 1) / a.e_chunk;
-        const int64_t parts = std::min<int64_t>(std::min<int64_t>(nbs, 64),
-                                                (two_waves + wx * chunks - 1) / (wx * chunks));
-        const MixedKernel wk = walk_kernel(acc, field_flags);
-        if (cudaFuncSetAttribute(wk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-            cudaSuccess)
-            return LW_ECUDA;
-        wk<<<dim3((unsigned)wx, (unsigned)chunks, (unsigned)parts), kMixThreads, smem, st>>>(a);
-        if (launch_status() != LW_OK) return LW_ECUDA;
-    }
     // static tables + double-buffered staging exceed the 48 KB default: opt in
     const MixedKernel kern = split ? mixed_kernel<true>(acc_of(precision), field_flags)
                                    : mixed_kernel<false>(acc_of(precision), field_flags);

@@ -1,4 +1,4 @@
-"""Which launch deposits a tile of the mixed deposit, and that it does not matter: the walk of dense
+"""Which way a tile of the mixed deposit is taken, and that it does not matter: the walk of dense
 tiles and the search add the same contributions, to the bit (a record of one electron has one
 contribution per bin, so no order of additions enters)."""
 import numpy as np
@@ -105,17 +105,19 @@ def _per_step(traj, n_hat, grid):
     return [float(adv[k:k + 512].mean()) / (grid.dt_u * traj.n_s) for k in range(0, len(adv), 512)]
 
 
-def _ms(call):
-    """Shortest of seven calls, by events on the stream."""
-    times = []
-    for _ in range(9):
-        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
-        a.record()
-        call()
-        b.record()
-        b.synchronize()
-        times.append(a.elapsed_time(b))
-    return min(times[2:])
+def _ms(*calls):
+    """Shortest of nine runs of each call, in turn, by events on the stream."""
+    best = [float("inf")] * len(calls)
+    for rep in range(11):
+        for n, call in enumerate(calls):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            call()
+            b.record()
+            b.synchronize()
+            if rep >= 2:
+                best[n] = min(best[n], a.elapsed_time(b))
+    return best
 
 
 def test_dense_tiles_are_walked():
@@ -130,18 +132,19 @@ def test_dense_tiles_are_walked():
     traj = lw.lw_trajectories_upload(tr.t, tr.r, tr.beta, tr.beta_dot)
     det = lw.Detector(n_hat)
     grid = _grid(traj, det, 12300)
-    assert [v > 1.0 for v in _per_step(traj, n_hat, grid)] == [False, True, True]
-    rec, _ = _deposit(traj, det, grid, lw.LW_MIXED_F32X4)
-    walked, first = _ms(lambda: _deposit(traj, det, grid, lw.LW_MIXED_F32X4)), rec.clone()
+    assert [v > 1.3 for v in _per_step(traj, n_hat, grid)] == [False, True, True]
+    first, _ = _deposit(traj, det, grid, lw.LW_MIXED_F32X4)
     other = _searched(traj)
-    moved = _ms(lambda: _deposit(other, det, grid, lw.LW_MIXED_F32X4))
+    walked, moved = _ms(lambda: _deposit(traj, det, grid, lw.LW_MIXED_F32X4),
+                        lambda: _deposit(other, det, grid, lw.LW_MIXED_F32X4))
     _span(traj).zero_()
     assert _per_step(traj, n_hat, grid) == [0.0, 0.0, 0.0]
-    searched = _ms(lambda: _deposit(traj, det, grid, lw.LW_MIXED_F32X4))
+    (searched,) = _ms(lambda: _deposit(traj, det, grid, lw.LW_MIXED_F32X4))
+    print(walked, moved, searched)
     assert walked < 0.8 * searched and walked < 0.8 * moved
     rec, _ = _deposit(traj, det, grid, lw.LW_MIXED_F32X4)
-    # FP32 additions of the same contributions in two orders; a tile deposited by both launches or by
-    # neither is an error of order one
+    # FP32 additions of the same contributions in two orders; a tile deposited twice or not at all
+    # is an error of order one
     assert (first - rec).abs().max() <= 1e-3 * rec.abs().max()
 
 
@@ -159,6 +162,7 @@ def test_a_bunch_is_not_slower_than_by_search(prec, per_step):
     grid = lw.grid_from_bounds(lo, hi, 1 << 16)
     (had,) = _per_step(traj, w.n_hat, grid)
     grid = lw.grid_from_bounds(lo, hi, int(per_step / had * (1 << 16)))
-    chosen = _ms(lambda: lw.lw_deposit_time_domain(traj, det, grid, prec))
-    searched = _ms(lambda: lw.lw_deposit_time_domain(other, det, grid, prec))
+    chosen, searched = _ms(lambda: lw.lw_deposit_time_domain(traj, det, grid, prec),
+                           lambda: lw.lw_deposit_time_domain(other, det, grid, prec))
+    print(chosen, searched)
     assert chosen <= 1.04 * searched
