@@ -69,14 +69,15 @@ struct DepositArgs {
     void* record;
     int32_t* status;
     int e_chunk;
-    const double* span;   // mixed: mean advance, or null where no tile can be dense (walk_tile)
+    const double* span;   // mixed: mean advance, or null where nothing is decided by it (tile_kind)
+    int walk;             // whether tiles may be dense
 };
 
 // Inputs whose advanced time need not increase from sample to sample: flagged by the upload (a step
 // longer than c0 dt, times out of order, non-finite values), or not known.
+constexpr int kIrregular = LW_ST_STEP | LW_ST_TIME | LW_ST_NONFINITE;
 __device__ __forceinline__ bool irregular(const DepositArgs& p) {
-    return !p.input_status ||
-           (*p.input_status & (LW_ST_STEP | LW_ST_TIME | LW_ST_NONFINITE)) != 0;
+    return !p.input_status || (*p.input_status & kIrregular) != 0;
 }
 
 // ------------------------------------------------------------------ FP64
@@ -585,6 +586,10 @@ template <int ACC>
 __host__ __device__ constexpr float walk_density() {
     return ACC == kAccF32X4 ? 1.3f : ACC == kAccF32 ? 1.6f : 1.9f;
 }
+// Grid points per step below which the blocks of a tile's electron are not divided over CTAs: starting
+// a CTA then costs more than its points (209 electrons x 3,239 steps x 779 pixels at 0.002 per step: 91 us
+// undivided, 98 in two parts; 450 electrons x 3,000 steps x 484 pixels at 2 per step: 2.1 and 1.6 ms).
+constexpr float kSparse = 0.01f;
 constexpr int kWalkTile = 512;  // pixels that share a decision
 constexpr int kWalkMap = 256;   // grid points of a segment mapped to steps at a time
 
@@ -678,15 +683,18 @@ __device__ __forceinline__ void walk_block(const float4* s_scan, const float4* s
     }
 }
 
-// Whether the electrons are walked for the 512 pixels around `pix`: the grid points per step that
-// the trajectories' mean advance (span, stored by the upload) gives the middle pixel.  A test of
-// every electron, by each CTA, cost more than it sorted out (36 FP64 instructions: 10 % of a
-// 1,001-electron step).
-__device__ __noinline__ bool walk_tile(const double* span, const double* n_hat, int64_t n_pix,
-                                       int64_t pix, double points, double inv_dtu) {
+// Grid points per step that the trajectories' mean advance (span, stored by the upload) gives the
+// middle pixel of the 512 around `pix`; NaN for irregular inputs, about which nothing is decided
+// (they are searched, undivided: where coordinates go back within a block, the walk's running maximum
+// and the search's bisection can end in different steps).  A test of every electron, by each CTA, cost
+// more than it sorted out (36 FP64 instructions: 10 % of a 1,001-electron step).
+__device__ __noinline__ float tile_points(const double* span, const double* n_hat, int64_t n_pix,
+                                          int64_t pix, double inv_dtu, double n_s,
+                                          const int32_t* input_status) {
+    const int status = *input_status;
     const double* n = n_hat + 3 * min(pix, n_pix - 1);
     const double nr = (n[0] * span[1] + n[1] * span[2]) - (1.0 - n[2]) * span[3];
-    return (span[0] - nr * kInvC0) * inv_dtu > points;
+    return (status & kIrregular) ? NAN : to_float((span[0] - nr * kInvC0) * inv_dtu) / (float)n_s;
 }
 
 // The work of one CTA: pixel tile `tile` (kMixThreads * PIX pixels) and electron
@@ -743,7 +751,6 @@ __device__ __forceinline__ int mixed_cta(const DepositArgs& p, int64_t tile, int
     constexpr int kSlots = kMixThreads * PIX;
     const int B = p.block;
     const size_t sbytes = stage_bytes(B);
-    constexpr int kWarpsMix = kMixThreads / 32;
     // Slot numbering: lane-major, wslot + lane * PIX + q for pixel q of a lane -- the
     // order in which the warp's jobs are listed, so that the 32 jobs of a round, which
     // mostly belong to consecutive slots, read consecutive per-slot records.
@@ -1472,15 +1479,24 @@ __global__ void __launch_bounds__(kFp64Threads) deposit_fp64_kernel(DepositArgs 
     block_status_or(p.status, bits);
 }
 
-// walk_tile for the CTA (thread 0 decides; out of line it keeps its registers).  Irregular inputs are searched: where coordinates go back
-// within a block, the walk's running maximum and the search's bisection can end in different steps.
+// What the CTA does with its tile, by its grid points per step (thread 0 decides; out of line it
+// keeps its registers)
+enum { kTileSparse = 0, kTileSearch = 1, kTileDense = 2 };
 template <int ACC>
-__device__ __forceinline__ bool tile_is_dense(const DepositArgs& p, int64_t pix0) {
-    int dense = 0;
-    if (threadIdx.x == 0 && !irregular(p))
-        dense = walk_tile(p.span, p.n_hat, p.n_pix, pix0 / kWalkTile * kWalkTile + kWalkTile / 2,
-                          walk_density<ACC>() * (double)(p.ns1 - 1), p.inv_dtu);
-    return __syncthreads_or(dense) != 0;
+__device__ __forceinline__ int tile_kind(const DepositArgs& p, int64_t pix0) {
+    __shared__ int s_kind;
+    if (threadIdx.x == 0) {
+        const float u = p.input_status
+                            ? tile_points(p.span, p.n_hat, p.n_pix,
+                                          pix0 / kWalkTile * kWalkTile + kWalkTile / 2, p.inv_dtu,
+                                          (double)(p.ns1 - 1), p.input_status)
+                            : NAN;
+        s_kind = p.walk && u > walk_density<ACC>() ? kTileDense
+                 : u < kSparse                     ? kTileSparse
+                                                   : kTileSearch;
+    }
+    __syncthreads();
+    return s_kind;
 }
 
 template <int PIX, int ACC, int FL, bool SPLIT>
@@ -1488,9 +1504,14 @@ __global__ void __launch_bounds__(kMixThreads, kMixMinBlocks) deposit_mixed_kern
     // the precision check launched after this grid (programmatic dependent launch) may
     // start once every CTA of this grid has started: it fills the SMs of the last wave
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int kind = p.span ? tile_kind<ACC>(p, (int64_t)blockIdx.x * (kMixThreads * PIX)) : kTileSearch;
+    int part = blockIdx.z, parts = gridDim.z;
+    if (SPLIT && kind == kTileSparse) {
+        if (part > 0) return;
+        parts = 1;
+    }
     int bits = 0;
-    if (ACC != kAccKahan && p.span &&
-        tile_is_dense<ACC>(p, (int64_t)blockIdx.x * (kMixThreads * PIX))) {
+    if (ACC != kAccKahan && kind == kTileDense) {
         // One pixel per thread (two spill 36 to 210 bytes, 11 % slower): the tile's halves in turn.
         // The same unit as the search's, so that electrons are added in the order in which they are
         // searched: an FP32 record is rounded at every addition, and units of four electrons instead
@@ -1502,12 +1523,10 @@ __global__ void __launch_bounds__(kMixThreads, kMixMinBlocks) deposit_mixed_kern
         for (int h = 0; h < PIX; ++h) {
             const int64_t tile = (int64_t)blockIdx.x * PIX + h;
             if (tile * kMixThreads < p.n_pix)
-                bits |= mixed_cta<1, ACC, FL, kWalk, SPLIT>(p, tile, blockIdx.y, blockIdx.z,
-                                                            gridDim.z);
+                bits |= mixed_cta<1, ACC, FL, kWalk, SPLIT>(p, tile, blockIdx.y, part, parts);
         }
     } else {
-        bits = mixed_cta<PIX, ACC, FL, kSearch, SPLIT>(p, blockIdx.x, blockIdx.y, blockIdx.z,
-                                                       gridDim.z);
+        bits = mixed_cta<PIX, ACC, FL, kSearch, SPLIT>(p, blockIdx.x, blockIdx.y, part, parts);
     }
     block_status_or(p.status, bits);
 }
@@ -1734,14 +1753,17 @@ extern "C" int lw_deposit_time_domain(const lw_traj* traj, const lw_detector* de
                            precision == LW_MIXED_F32X4 ? kMixMaxChunkX4 : kMixMaxChunk);
     a.e_chunk = (int)std::max<int64_t>(ec, (traj->n_e + 65534) / 65535);
     dim3 g((unsigned)tiles, (unsigned)((traj->n_e + a.e_chunk - 1) / a.e_chunk));
-    // less than two waves of CTAs: tiles of one pixel per thread, and the blocks of an electron
-    // divided over grid z, up to two waves (16 electrons x 2,000 steps x 1,024 pixels: 571 us in 32
-    // CTAs, 110 in 256)
+    // Few CTAs: tiles of one pixel per thread, and the blocks of an electron divided over grid z (unless
+    // the tile turns out sparse), up to two waves (16 electrons x 2,000 steps x 1,024 pixels: 571 us in
+    // 32 CTAs, 110 in 256).  Few is less than 1.6 waves, or than two where the smaller tiles are no
+    // more of them: at 1.6 to 2 waves the last one is full enough, and halved tiles stage every
+    // sample twice (450 electrons x 1,969 steps x 780 pixels, 900 CTAs: 55 us, halved 65).
     const int64_t nbs = (traj->n_s - 1) / traj->block + 1;
-    const int64_t two_waves = (int64_t)kSms * kMixMinBlocks * 2;
-    const bool split = (int64_t)g.x * g.y < two_waves;
+    const int64_t two_waves = (int64_t)kSms * kMixMinBlocks * 2, ctas2 = (int64_t)g.x * g.y;
+    const int64_t tiles1 = (det->n_pix + kMixThreads - 1) / kMixThreads;
+    const bool split = 5 * ctas2 < 4 * two_waves || (ctas2 < two_waves && tiles1 == tiles);
     if (split) {
-        g.x = (unsigned)((det->n_pix + kMixThreads - 1) / kMixThreads);
+        g.x = (unsigned)tiles1;
         const int64_t ctas = (int64_t)g.x * g.y;
         g.z = (unsigned)std::min<int64_t>(std::min<int64_t>(nbs, 64), (two_waves + ctas - 1) / ctas);
     }
@@ -1751,8 +1773,8 @@ extern "C" int lw_deposit_time_domain(const lw_traj* traj, const lw_detector* de
     const int acc = acc_of(precision);
     const float density = acc == kAccF32X4 ? walk_density<kAccF32X4>()
                           : acc == kAccF32 ? walk_density<kAccF32>() : walk_density<kAccF64>();
-    if (acc != kAccKahan && (double)grid->n_bins > (double)density * (double)traj->n_s)
-        a.span = traj_span(traj);
+    a.walk = acc != kAccKahan && (double)grid->n_bins > (double)density * (double)traj->n_s;
+    if (a.walk || g.z > 1) a.span = traj_span(traj);
     // static tables + double-buffered staging exceed the 48 KB default: opt in
     const MixedKernel kern = split ? mixed_kernel<true>(acc_of(precision), field_flags)
                                    : mixed_kernel<false>(acc_of(precision), field_flags);

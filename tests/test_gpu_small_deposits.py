@@ -1,6 +1,7 @@
-"""Deposits of a bunch whose grid could hold as many points per step as the walk's lines say and does
-not: what decides that costs next to nothing.  Beside the same deposit with a view whose order stands
-elsewhere, which has no mean advance and decides nothing."""
+"""Small deposits of a bunch, far fewer grid points than steps.  Where the grid could hold as many per
+step as the walk's lines say, what decides that costs next to nothing; few electrons' blocks are not
+divided over CTAs.  Beside the same deposit with a view whose order stands elsewhere, which has no mean
+advance and decides nothing."""
 import numpy as np
 import pytest
 
@@ -12,14 +13,12 @@ from workloads import simple  # noqa: E402
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n_e,n_s,n_pix,n_bins", [(226, 1855, 714, 9686), (926, 1523, 984, 7492),
-                                                  (2900, 1050, 799, 4100)])
-@pytest.mark.parametrize("prec", [lw.LW_MIXED, lw.LW_MIXED_F32, lw.LW_MIXED_F32X4])
-def test_sparse_tiles_cost_no_launch(n_e, n_s, n_pix, n_bins, prec):
+def _times(n_e, n_s, n_pix, n_bins, prec, spread):
+    """Shortest times [ms] of the deposit and of the one that decides nothing."""
     tr = simple.transverse_oscillation(n_e, n_s, 1e-17, 0.999, 0.002, 97.0, seed=n_e)
-    # arrivals spread over 500 times an electron's own span
+    # arrivals spread over many times an electron's own span
     own = n_s * 1e-17 * 1e-3
-    shift = np.linspace(0.0, 500 * own * 299792458.0, n_e)
+    shift = np.linspace(0.0, spread * own * 299792458.0, n_e)
     tr = simple.Trajectories(tr.t, tr.r - shift[:, None, None] * np.array([0.0, 0.0, 1.0]), tr.beta,
                              tr.beta_dot)
     rng = np.random.Generator(np.random.PCG64(1))
@@ -46,4 +45,18 @@ def test_sparse_tiles_cost_no_launch(n_e, n_s, n_pix, n_bins, prec):
             if rep >= 2:
                 best[n] = min(best[n], a.elapsed_time(b) / 50)
     print(best)
-    assert best[0] <= 1.04 * best[1] + 1e-3   # (a launch and a row of CTAs that end at once: 5 to 15 us)
+    return best
+
+
+@pytest.mark.parametrize("n_e,n_s,n_pix,n_bins", [(226, 1855, 714, 9686), (926, 1523, 984, 7492),
+                                                  (2900, 1050, 799, 4100)])
+@pytest.mark.parametrize("prec", [lw.LW_MIXED, lw.LW_MIXED_F32, lw.LW_MIXED_F32X4])
+def test_sparse_tiles_cost_no_launch(n_e, n_s, n_pix, n_bins, prec):
+    chosen, undecided = _times(n_e, n_s, n_pix, n_bins, prec, 500)
+    assert chosen <= 1.04 * undecided + 1e-3   # (a row of CTAs that end at once: 5 to 15 us)
+
+
+def test_sparse_tiles_of_few_electrons():
+    """209 electrons, whose blocks a denser tile's would be divided: 0.003 points per step."""
+    chosen, divided = _times(209, 3239, 779, 25345, lw.LW_MIXED_F32, 3000)
+    assert chosen <= 1.01 * divided + 1e-3
