@@ -10,22 +10,21 @@
 // an electron are listed and taken one per thread, each searching its step among
 // the stored samples; where they are many, and for trajectories out of order, a
 // thread owns a pixel and takes every step from staged blocks of samples.  Every
-// result of the time map, the bin index,
-// the field and the weights is the correctly rounded one of the operation order
-// documented in lw.h, so advanced times, bin indices and per-sample contributions
-// are bit-identical to a plain C loop without FMA contraction; only the order of
-// the atomic additions differs.
+// result of the time map, the bin index, the field and the weights is the correctly
+// rounded one of the operation order documented in lw.h, so advanced times, bin
+// indices and per-sample contributions are bit-identical to a plain C loop without
+// FMA contraction; only the order of the atomic additions differs.
 //
 // Mixed path: a thread owns one or two pixels and the electron's samples are staged
-// block by block in shared memory, once per CTA.  The bin coordinate u = (t_a - t_min)/dt_u is anchored once per
-// block of samples in double-FP32 arithmetic (integer part + FP32 fraction)
-// and evaluated per sample with three FP32 FMAs of small, block-relative
-// quantities.  Because t_a increases along a subluminal trajectory, a block
-// needs one coordinate per pixel (its last sample) to know which grid points
-// it reaches; each grid point's step is then found by a bracketed search
+// block by block in shared memory, once per CTA.  The bin coordinate
+// u = (t_a - t_min)/dt_u is anchored once per block of samples in double-FP32
+// arithmetic (integer part + FP32 fraction) and evaluated per sample with three FP32
+// FMAs of small, block-relative quantities.  Because t_a increases along a subluminal
+// trajectory, a block needs one coordinate per pixel (its last sample) to know which grid
+// points it reaches; each grid point's step is then found by a bracketed search
 // (regula falsi, then bisection) over the staged block, or, where grid points are as
-// many as steps, the block is walked sample by sample.  The field is FP32 in
-// the stable form
+// many as steps, the block is walked sample by sample.  The field is FP32 in the
+// stable form
 //   D = (1 - n_z) + n_z (1 - beta_z) - n_perp . beta_perp,
 // and contributions are added with FP64 atomics, a compensated pair of FP32
 // atomics, or FP32 atomics (the three mixed records).

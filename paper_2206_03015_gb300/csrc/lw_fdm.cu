@@ -14,12 +14,13 @@
 // frequency that leaves one complex product and six FMAs; partial sums over 16 samples are FP32
 // and are added to compensated (two-float) totals.
 //
-// Bound: the FP32 pipe (10 operations per sample and frequency, 42 more per 16 samples).  The rest
-// is kept off it or beside it: two warps of a CTA do the FP64 part ahead of the others through a
-// ring of groups of 32 samples (an FP64 instruction holds a warp for 64 cycles), a CTA takes two
-// blocks of frequencies so that they share it, two frequencies go into one packed FP32x2
-// instruction, and the CTAs of a cluster divide the samples and add their totals through
-// distributed shared memory, so that few pixels fill the GPU.  64 electrons x 1,000 steps x 144
+// Bound: the FP32 pipe, busy 66 % of the active cycles, beside instruction issue at 56 %
+// (32 electrons x 1,000 steps x 144 pixels x 2,048 frequencies; 10 operations per sample and
+// frequency, 42 more per 16 samples).  The rest is kept off it or beside it: two warps of a CTA do
+// the FP64 part ahead of the others through a ring of groups of 32 samples (an FP64 instruction
+// holds a warp for 64 cycles), a CTA takes two blocks of frequencies so that they share it, two
+// frequencies go into one packed FP32x2 instruction, and the CTAs of a cluster divide the samples
+// and add their totals through distributed shared memory, so that few pixels fill the GPU.  64 electrons x 1,000 steps x 144
 // pixels x 2,048 frequencies: 21.0 ms (16 threads per CTA doing the FP64 part between barriers)
 // -> 11.1 ms.
 #include <cooperative_groups.h>

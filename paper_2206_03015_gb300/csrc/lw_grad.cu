@@ -388,7 +388,8 @@ __global__ void __launch_bounds__(kAdjThreads) adj_deposit_kernel(AdjArgs p) {
 // relative to the step's first grid point, the sums over grid points and the per-sample
 // chain rule.  The record gradient enters scaled by a power of two 2^-e (|values| < 2,
 // e from its largest magnitude), so that its products with fields of up to ~1e30 /s stay
-// in FP32 range; the warp sums are unscaled in FP64 before the FP64 atomics.
+// in FP32 range; the warp sums are added to per-sample FP32 sums, which a last pass unscales
+// in FP64 into the caller's gradients.
 
 // largest |dL/drec| as ordered bits (non-negative doubles compare as integers)
 __global__ void adj_absmax_kernel(const double* __restrict__ R, int64_t n,
